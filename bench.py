@@ -293,7 +293,7 @@ def run_ours(args, world, rank, local):
                                    f"128 FP32 lanes / (2d+2) FP32 operations per feature",
                      "kernel_pipe_peak": pipe_peak, "kernel_pipe_frac": achieved / pipe_peak},
         "clocks": clk.summary(),
-        # per step: centre table, 7 kernels of the spatial sort, the morph kernel
+        # per step: the ordered centre table, 7 kernels of the samples' sort, the morph kernel
         "gpu_launches": args.steps * LAUNCHES_PER_MORPH,
         "wall_s_timed": wall1 - wall0,
     }

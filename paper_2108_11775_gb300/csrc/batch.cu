@@ -5,7 +5,7 @@
 // a list of (environment, tile) work units ordered longest first -- cost
 // M_e * T_e per tile -- are copied into the caller's workspace.
 // Run (launch-only, so a CUDA graph can capture it): every environment's
-// centre table, one spatial sort over all environments' samples (cell keys
+// ordered centre table, one spatial sort over all environments' samples (cell keys
 // are environment-major, so each environment's samples stay contiguous in
 // sorted order), then one persistent kernel whose blocks claim work units from
 // an atomic counter and run them with the same per-tile code as the
@@ -28,11 +28,12 @@ struct BatchEnv {        // device table entry (64-bit aligned)
   const float* x0;
   float* xT;
   float4* tab;
+  float4* box;
   int64_t N, M;
   int64_t sample_base;   // first global sample index (= first sorted position)
-  int64_t centre_base;   // first global centre index
   int64_t cell_base;     // first global cell key
-  int32_t d, T, bits, pad;
+  int32_t d, T, bits;    // bits, cbits: the grids of the samples' and the centres' order
+  int32_t cbits;
   float gamma, bias, eta, pad2;
 };
 
@@ -60,21 +61,24 @@ __device__ __forceinline__ int find_env(const int64_t* __restrict__ base, int n,
   return lo;
 }
 
-__global__ void k_batch_tables(const BatchEnv* __restrict__ envs, const int64_t* __restrict__ cbase, int n_envs,
-                               int64_t total_M) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total_M) return;
-  const int e = find_env(cbase, n_envs, g);
-  const BatchEnv& E = envs[e];
-  const int64_t m = g - E.centre_base;
-  const float wm = E.w[m];
-  const float lw = wm != 0.0f ? log2f(fabsf(wm)) : -INFINITY;
-  const float sg = wm > 0.0f ? 1.0f : (wm < 0.0f ? -1.0f : 0.0f);
-  if (E.d == 2) {
-    E.tab[m] = make_float4(E.centres[m * 2], E.centres[m * 2 + 1], lw, sg);
-  } else {
-    E.tab[2 * m] = make_float4(E.centres[m * 3], E.centres[m * 3 + 1], E.centres[m * 3 + 2], lw);
-    E.tab[2 * m + 1] = make_float4(sg, 0.0f, 0.0f, 0.0f);
+// One cluster per environment: its centres ordered, with their table and
+// group boxes (chunk by chunk, as the single-field launch's clusters do).
+__global__ void __cluster_dims__(kOrderBlocks, 1, 1) __launch_bounds__(kOrderThreads)
+    k_batch_tables(const BatchEnv* __restrict__ envs) {
+  __shared__ OrderSmem s;
+  const BatchEnv& E = envs[blockIdx.x / kOrderBlocks];
+  const int crank = (int)(blockIdx.x % kOrderBlocks);
+  for (int64_t m0 = 0; m0 < E.M; m0 += kOrderChunk) {
+    const int n = (int)min64(kOrderChunk, E.M - m0);
+    float4* box = E.box + m0 / kGroup * kGroupBox;
+    if (E.d == 2) {
+      const int share = cluster_order<2>(E.centres + m0 * 2, n, E.cbits, s, crank);
+      order_table<2>(E.centres + m0 * 2, E.w + m0, n, s, crank * share, share, E.tab + m0, box, nullptr, 0);
+    } else {
+      const int share = cluster_order<3>(E.centres + m0 * 3, n, E.cbits, s, crank);
+      order_table<3>(E.centres + m0 * 3, E.w + m0, n, s, crank * share, share, E.tab + 2 * m0, box, nullptr, 0);
+    }
+    cluster_barrier();   // the order is read before the next chunk's
   }
 }
 
@@ -172,6 +176,8 @@ k_morph_batched(const BatchEnv* __restrict__ envs, const BatchUnit* __restrict__
     const BatchEnv& E = envs[un.env];
     TileArgs a;
     a.tab = E.tab;
+    a.box = E.box;
+    a.ngroups = group_count(E.M);
     a.M = E.M;
     a.gamma = E.gamma;
     a.bias = E.bias;
@@ -198,16 +204,16 @@ k_morph_batched(const BatchEnv* __restrict__ envs, const BatchUnit* __restrict__
 }
 
 template <int W, int K>
-static size_t batched_smem() {
-  const size_t a = fast_smem_bytes<2, W, K>(), b = fast_smem_bytes<3, W, K>();
-  return a > b ? a : b;
+static size_t batched_smem(int64_t max_M) {
+  const size_t a = tile_smem_bytes<2, W, K>(), b = tile_smem_bytes<3, W, K>();
+  return (a > b ? a : b) + near_bytes(max_M);
 }
 
 // ---------------------------------------------------------------- layout
 struct BatchLayout {
-  size_t off_counter, off_envs, off_sbase, off_cbase, off_units, off_boxes, off_tabs, off_keys, off_perm, off_counts,
+  size_t off_counter, off_envs, off_sbase, off_units, off_boxes, off_tabs, off_keys, off_perm, off_counts,
       off_offs, off_cursor, off_chunks, bytes;
-  std::vector<size_t> tab_off;
+  std::vector<size_t> tab_off, box_off;
   int64_t n_units, total_N, total_M, total_cells, nchunks;
 };
 
@@ -232,12 +238,15 @@ static BatchLayout batch_layout(const pdmp_env* envs, int n, int variant) {
   L.off_counter = take(16);
   L.off_envs = take(sizeof(BatchEnv) * n);
   L.off_sbase = take(sizeof(int64_t) * (n + 1));
-  L.off_cbase = take(sizeof(int64_t) * (n + 1));
   L.off_units = take(sizeof(BatchUnit) * L.n_units);
   L.off_boxes = take(sizeof(uint32_t) * 6 * n);
   L.tab_off.resize(n);
+  L.box_off.resize(n);
   L.off_tabs = p;
-  for (int e = 0; e < n; ++e) L.tab_off[e] = take((size_t)envs[e].field.M * 16 * (envs[e].field.d == 2 ? 1 : 2));
+  for (int e = 0; e < n; ++e) {
+    L.tab_off[e] = take((size_t)envs[e].field.M * 16 * (envs[e].field.d == 2 ? 1 : 2));
+    L.box_off[e] = take((size_t)group_count(envs[e].field.M) * kGroupBox * sizeof(float4));
+  }
   L.off_keys = take(sizeof(uint32_t) * L.total_N);
   L.off_perm = take(sizeof(int32_t) * L.total_N);
   L.off_counts = take(sizeof(uint32_t) * L.total_cells);
@@ -258,8 +267,8 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   const int tile = variant_tile(variant);
   char* base = (char*)ws;
   std::vector<BatchEnv> tab(n);
-  std::vector<int64_t> sb(n + 1), cb(n + 1);
-  int64_t s = 0, c = 0, cell = 0;
+  std::vector<int64_t> sb(n + 1);
+  int64_t s = 0, cell = 0, max_M = 1;
   for (int e = 0; e < n; ++e) {
     const pdmp_env& E = envs[e];
     BatchEnv& B = tab[e];
@@ -269,25 +278,24 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
     B.x0 = E.x0;
     B.xT = E.xT;
     B.tab = (float4*)(base + L.tab_off[e]);
+    B.box = (float4*)(base + L.box_off[e]);
     B.N = E.N;
     B.M = E.field.M;
     B.sample_base = s;
-    B.centre_base = c;
     B.cell_base = cell;
     B.d = E.field.d;
     B.T = E.T;
     B.bits = sort_bits(E.field.d, E.N);
+    B.cbits = sort_bits(E.field.d, std::min<int64_t>(E.field.M, kOrderChunk));
+    max_M = std::max(max_M, E.field.M);
     B.gamma = E.field.gamma;
     B.bias = E.field.bias;
     B.eta = E.eta;
     sb[e] = s;
-    cb[e] = c;
     s += E.N;
-    c += E.field.M;
     cell += (int64_t)1 << (B.d * B.bits);
   }
   sb[n] = s;
-  cb[n] = c;
   // work units, longest first (cost M T per tile), then by environment and tile
   std::vector<BatchUnit> units;
   units.reserve(L.n_units);
@@ -301,8 +309,6 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   if ((e = cudaMemcpyAsync(base + L.off_envs, tab.data(), sizeof(BatchEnv) * n, cudaMemcpyHostToDevice, st)))
     return e;
   if ((e = cudaMemcpyAsync(base + L.off_sbase, sb.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st)))
-    return e;
-  if ((e = cudaMemcpyAsync(base + L.off_cbase, cb.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st)))
     return e;
   if (!units.empty() &&
       (e = cudaMemcpyAsync(base + L.off_units, units.data(), sizeof(BatchUnit) * units.size(),
@@ -318,7 +324,7 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   int block = 32 * kVariantW[variant];
 #define PDMP_VARIANT(V, W_, K_)                                                                                      \
   if (variant == V) {                                                                                                \
-    smem = batched_smem<W_, K_>();                                                                                   \
+    smem = batched_smem<W_, K_>(max_M);                                                                               \
     if ((e = cudaFuncSetAttribute(k_morph_batched<W_, K_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) \
       return e;                                                                                                      \
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_morph_batched<W_, K_>, block, smem))) return e; \
@@ -342,7 +348,7 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   plan->off[0] = L.off_counter;
   plan->off[1] = L.off_envs;
   plan->off[2] = L.off_sbase;
-  plan->off[3] = L.off_cbase;
+  plan->off[3] = 0;   // unused
   plan->off[4] = L.off_units;
   plan->off[5] = L.off_boxes;
   plan->off[6] = L.off_keys;
@@ -360,7 +366,6 @@ cudaError_t batch_run(const pdmp_batch_plan* P, void* ws, cudaStream_t st) {
   auto at = [&](int i) { return base + P->off[i]; };
   const BatchEnv* envs = (const BatchEnv*)at(1);
   const int64_t* sbase = (const int64_t*)at(2);
-  const int64_t* cbase = (const int64_t*)at(3);
   const BatchUnit* units = (const BatchUnit*)at(4);
   uint32_t* boxes = (uint32_t*)at(5);
   uint32_t* keys = (uint32_t*)at(6);
@@ -373,8 +378,7 @@ cudaError_t batch_run(const pdmp_batch_plan* P, void* ws, cudaStream_t st) {
   const int n = P->n_envs;
   cudaError_t e;
   if ((e = cudaMemsetAsync(counter, 0, 16, st))) return e;
-  if (P->total_M > 0)
-    k_batch_tables<<<(unsigned)((P->total_M + 255) / 256), 256, 0, st>>>(envs, cbase, n, P->total_M);
+  k_batch_tables<<<(unsigned)n * kOrderBlocks, kOrderThreads, 0, st>>>(envs);
   if (P->total_N > 0) {
     k_batch_init_boxes<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(boxes, n);
     if ((e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * P->total_cells, st))) return e;

@@ -3,6 +3,7 @@
 //
 #pragma once
 #include "field.cuh"
+#include "order.cuh"
 
 namespace pdmp {
 
@@ -65,7 +66,8 @@ __device__ __forceinline__ u64 ex2x2_neg(u64 a) {
 // Tile shape: W warps per block (each summing over its share of M) and K
 // samples per lane (even: f32x2 pairs).  The single-field launch uses
 // W = 4, K = 10 (measured fastest on the 2-D fitted workload among K = 6..16,
-// W = 2..8, unroll 1..4 and 32..128-centre stages); the batched launch picks
+// W = 2..8, unroll 1..4; 32-centre stages cost 1 % against 64 and make the
+// groups that a tile can leave out smaller); the batched launch picks
 // among a few shapes (autotuned).  Shapes with K > 8 need more than 128
 // registers a thread and run 12 warps per SM, the others 16.
 // The expanded exponent a_m + b_m . u carries a rounding error of about
@@ -76,12 +78,13 @@ __device__ __forceinline__ u64 ex2x2_neg(u64 a) {
 #define PDMP_EXPAND_LIMIT 8.0f
 #endif
 #ifndef PDMP_WARP_STAGE
-#define PDMP_WARP_STAGE 64
+#define PDMP_WARP_STAGE 32
 #endif
 #ifndef PDMP_FAST_UNROLL
 #define PDMP_FAST_UNROLL 2
 #endif
 constexpr int kWarpStage = PDMP_WARP_STAGE;    // centres per warp per shared-memory stage
+static_assert(kWarpStage == kGroup, "a stage is one group of ordered centres");
 constexpr int kFastUnroll = PDMP_FAST_UNROLL;  // centres per unrolled inner iteration
 
 template <int W, int K>
@@ -125,23 +128,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// table: RBF centre records {mu_0 .. mu_{d-1}, lw = log2|w|, sg = sign(w)}
-template <int D>
-__global__ void k_rbf_table(const float* __restrict__ centres, const float* __restrict__ w, int64_t M,
-                            float4* __restrict__ tab) {
-  int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M) return;
-  float wm = w[m];
-  float lw = wm != 0.0f ? log2f(fabsf(wm)) : -INFINITY;
-  float sg = wm > 0.0f ? 1.0f : (wm < 0.0f ? -1.0f : 0.0f);
-  if (D == 2) {
-    tab[m] = make_float4(centres[m * 2], centres[m * 2 + 1], lw, sg);
-  } else {
-    tab[2 * m] = make_float4(centres[m * 3], centres[m * 3 + 1], centres[m * 3 + 2], lw);
-    tab[2 * m + 1] = make_float4(sg, 0.0f, 0.0f, 0.0f);
-  }
-}
 
 // One warp copies the table entries of centres [m0, m0 + kWarpStage) into
 // its raw buffer (asynchronously; each lane copies the entries it later
@@ -226,7 +212,9 @@ __device__ __forceinline__ void stage_build(int64_t M, int64_t m0, bool expanded
 // position to a sample index; the sample's index in x0 / xT / ckpt / traj /
 // steps is perm[p] - perm_base, and those arrays hold N samples.
 struct TileArgs {
-  const float4* tab;
+  const float4* tab;     // centre table in the order of rbf_order
+  const float4* box;     // its groups' boxes
+  int ngroups;
   int64_t M;
   float gamma, bias, eta;
   int T;
@@ -276,6 +264,100 @@ __device__ __forceinline__ bool tile_frame(const float (&x)[K][D], const bool (&
   return expanded;
 }
 
+// ------------------------------------------------------------- near groups
+// A group of centres is far from a tile at a state when every one of its
+// features is exactly zero for every sample there (see rbf_order.cu): with d
+// the distance between the two boxes, the exponents the kernels form are at
+// most lw_max - g' d^2 (the expanded form's + g' R^2, its factor f = 2^(-g'
+// |u|^2) taken out), and ex2.approx.ftz returns 0 below -126.  One unit more
+// covers the rounding of the exponents and of this test.  A tile with a
+// sample that is not finite has no far groups (its sums must reach it).
+//
+// The near groups are marked in shared memory, one bit each, by all warps of
+// the block together once per sweep; groups past kNearWords * 32 (M > 2^20)
+// count as near.  Every warp then walks the marked groups that are its own.
+constexpr int kNearWords = 1024;
+
+__host__ __device__ __forceinline__ int near_words(int ngroups) {
+  const int n = (ngroups + 31) / 32;
+  return n < kNearWords ? n : kNearWords;
+}
+__host__ __device__ __forceinline__ size_t near_bytes(int64_t M) {
+  return ((size_t)near_words(group_count(M)) * 4 + 15) & ~size_t(15);
+}
+
+// Marks the groups that are near the tile's box [lo, hi] (of x, the same in
+// every warp); a block barrier before and after must separate it from the
+// walks of the sweep before and of this one.  unweighted: sums in which phi
+// stands without its weight; all: mark every group.
+template <int D, int W, int K>
+__device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ngroups, const float (&x)[K][D],
+                                          const bool (&act)[K], const float (&lo)[D], const float (&hi)[D],
+                                          bool expanded, float gl2e, bool unweighted, bool all, uint32_t* words,
+                                          int warp, int lane) {
+  float R2 = 0.0f;
+  bool odd = false;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const float h = 0.5f * (hi[j] - lo[j]);
+    R2 = fmaf(h, h, R2);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int j = 0; j < D; ++j) odd = odd || (act[k] && !(fabsf(x[k][j]) < INFINITY));
+  odd = __any_sync(0xffffffffu, odd);
+  const float lim = odd || all ? INFINITY : 127.0f + (expanded ? gl2e * R2 : 0.0f);
+  const int nw = near_words(ngroups);
+  for (int q = warp; q < nw; q += W) {
+    const int g = q * 32 + lane;
+    bool near = false;
+    if (g < ngroups) {
+      const float4 b0 = box[kGroupBox * g], b1 = box[kGroupBox * g + 1];
+      const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
+      float d2 = 0.0f;
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        const float gap = fmaxf(0.0f, fmaxf(blo[j] - hi[j], lo[j] - bhi[j]));
+        d2 = fmaf(gap, gap, d2);
+      }
+      near = !(fmaf(gl2e, d2, -(unweighted ? fmaxf(b0.w, 0.0f) : b0.w)) > lim);
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, near);
+    if (lane == 0) words[q] = m;
+  }
+}
+
+// The near groups number own, own + stride, own + 2 stride, ... in order.
+struct NearWalk {
+  const uint32_t* words;
+  int ngroups, stride, skip, q;
+  uint32_t m;
+  __device__ __forceinline__ NearWalk(const uint32_t* w, int ng, int own, int st)
+      : words(w), ngroups(ng), stride(st), skip(own), q(-1), m(0) {}
+  // the next one, or -1 (the same in every lane)
+  __device__ __forceinline__ int next() {
+    for (;;) {
+      const int pc = __popc(m);
+      if (pc > skip) {
+        for (; skip > 0; --skip) m &= m - 1;
+        const int b = __ffs(m) - 1;
+        m &= m - 1;
+        skip = stride - 1;
+        return q * 32 + b;
+      }
+      skip -= pc;
+      if (++q * 32 >= ngroups) {
+        q -= 1;
+        m = 0;
+        return -1;
+      }
+      const int left = ngroups - q * 32;
+      m = q < kNearWords ? words[q] : (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
+    }
+  }
+};
+
 // Adds the kWarpStage staged records rec to the pair sums S, G of this lane's
 // samples (U: the samples relative to the origin, packed in pairs).
 template <int D, int P>
@@ -283,7 +365,7 @@ __device__ __forceinline__ void stage_accumulate(const u64* rec, bool expanded, 
                                                  u64 (&S)[P], u64 (&G)[P][D]) {
   constexpr int RP = FastRec<D>::kPairs;
   if (expanded) {
-#pragma unroll kFastUnroll
+#pragma unroll (P <= 2 ? 4 : kFastUnroll)
     for (int c = 0; c < kWarpStage; ++c) {
       const ulonglong2* q = reinterpret_cast<const ulonglong2*>(rec + (size_t)c * RP);
       u64 r[RP];
@@ -314,7 +396,7 @@ __device__ __forceinline__ void stage_accumulate(const u64* rec, bool expanded, 
     }
   } else {
     const u64 ng = pk(-gl2e, -gl2e);
-    for (int c = 0; c < kWarpStage; ++c) {
+    auto one = [&](int c) {
       const u64* r = rec + (size_t)c * RP;
 #pragma unroll
       for (int i = 0; i < P; ++i) {
@@ -329,6 +411,12 @@ __device__ __forceinline__ void stage_accumulate(const u64* rec, bool expanded, 
 #pragma unroll
         for (int j = 0; j < D; ++j) G[i][j] = fma2(we, dx[j], G[i][j]);
       }
+    };
+    if constexpr (P <= 2) {   // few pairs: more centres in flight
+#pragma unroll 4
+      for (int c = 0; c < kWarpStage; ++c) one(c);
+    } else {
+      for (int c = 0; c < kWarpStage; ++c) one(c);
     }
   }
 }
@@ -388,7 +476,7 @@ template <int D, int P>
 __device__ __forceinline__ void stage_accumulate_origin(const u64* rec, const u64 (&U)[P][D], u64 (&S)[P],
                                                         u64 (&G)[P][D]) {
   constexpr int RP = FastRec<D>::kPairs;
-  for (int c = 0; c < kWarpStage; ++c) {
+  auto one = [&](int c) {
     const u64* r = rec + (size_t)c * RP;
 #pragma unroll
     for (int i = 0; i < P; ++i) {
@@ -403,6 +491,12 @@ __device__ __forceinline__ void stage_accumulate_origin(const u64* rec, const u6
 #pragma unroll
       for (int j = 0; j < D; ++j) G[i][j] = fma2(e, r[D + 2 + j], G[i][j]);
     }
+  };
+  if constexpr (P <= 2) {
+#pragma unroll 4
+    for (int c = 0; c < kWarpStage; ++c) one(c);
+  } else {
+    for (int c = 0; c < kWarpStage; ++c) one(c);
   }
 }
 
@@ -420,93 +514,114 @@ __device__ __forceinline__ void tile_load(const TileArgs& a, int64_t p0, int64_t
   }
 }
 
+// End of step t for sample k of this lane: the Euler update of Eq. (1) from
+// the totals acc = (S, G) of its sums; the writer (one warp of the tile) also
+// writes the trace and the last logit and gradient.
+template <int D, int K, bool TRACE>
+__device__ __forceinline__ void tile_update(const TileArgs& a, int t, int64_t p0, const bool (&act)[K],
+                                            float (&x)[K][D], const float (&o)[D], bool expanded, const float4& acc,
+                                            int k, bool writer, int lane) {
+  const int64_t N = a.N;
+  const float gamma = a.gamma, bias = a.bias, eta = a.eta;
+  const int T = a.T;
+  const float gl2e = gamma * kLog2e;
+  const float Ssum = acc.x, Gs[3] = {acc.y, acc.z, acc.w};
+  float shat, ghat[D];
+  if (expanded) {
+    float u[D], u2 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      u[j] = x[k][j] - o[j];
+      u2 = fmaf(u[j], u[j], u2);
+    }
+    const float f = ex2_approx(-gl2e * u2);
+    shat = f * Ssum;
+#pragma unroll
+    for (int j = 0; j < D; ++j) ghat[j] = f * fmaf(u[j], Ssum, -Gs[j]);
+  } else {
+    shat = Ssum;
+#pragma unroll
+    for (int j = 0; j < D; ++j) ghat[j] = Gs[j];
+  }
+  float d1, d2;
+  sigmoid_d12(shat + bias, d1, d2);
+  const float c = -eta * d1;
+  const int64_t p = p0 + k * 32 + lane;
+  const bool own = act[k] && writer;
+  const bool last_out = t == T - 1 && (a.s_out != nullptr || a.g_out != nullptr);
+  const int64_t n = (own && (TRACE || last_out)) ? (int64_t)a.perm[p] - a.perm_base : 0;
+  if (own && a.s_out != nullptr && t == T - 1) a.s_out[n] = shat + bias;
+  if (own && a.g_out != nullptr && t == T - 1)
+#pragma unroll
+    for (int j = 0; j < D; ++j) a.g_out[n * D + j] = d1 * (-2.0f * gamma * ghat[j]);
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const float inc = __fmul_rn(c, -2.0f * gamma * ghat[j]);
+    if (TRACE && act[k] && writer) {
+      a.traj[((int64_t)t * N + n) * D + j] = x[k][j];
+      a.steps[((int64_t)t * N + n) * D + j] = inc;
+    }
+    x[k][j] = __fadd_rn(x[k][j], inc);
+  }
+}
+
+// The checkpoint after step t, if one is due (called by the writer warp).
+template <int D, int K>
+__device__ __forceinline__ void tile_checkpoint(const TileArgs& a, int t, int64_t p0, const bool (&act)[K],
+                                                const float (&x)[K][D], int lane) {
+  if (a.ckpt == nullptr || (t + 1) % a.kck != 0) return;
+  float* dst = a.ckpt + (int64_t)((t + 1) / a.kck - 1) * a.N * D;
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (act[k]) {
+      const int64_t n = (int64_t)a.perm[p0 + k * 32 + lane] - a.perm_base;
+#pragma unroll
+      for (int j = 0; j < D; ++j) dst[n * D + j] = x[k][j];
+    }
+}
+
+// Writes one warp's sums of the tile's samples to dst (32 K float4s).
+template <int D, int K>
+__device__ __forceinline__ void tile_put_sums(const u64 (&S)[K / 2], const u64 (&G)[K / 2][D], float4* dst, int lane) {
+#pragma unroll
+  for (int i = 0; i < K / 2; ++i) {
+    float s0, s1, g0[D], g1[D];
+    upk(S[i], s0, s1);
+#pragma unroll
+    for (int j = 0; j < D; ++j) upk(G[i][j], g0[j], g1[j]);
+    dst[(2 * i) * 32 + lane] = make_float4(s0, g0[0], g0[1], D == 3 ? g0[D - 1] : 0.0f);
+    dst[(2 * i + 1) * 32 + lane] = make_float4(s1, g1[0], g1[1], D == 3 ? g1[D - 1] : 0.0f);
+  }
+}
+
+__device__ __forceinline__ void add4(float4& acc, const float4& b) {
+  acc.x += b.x;
+  acc.y += b.y;
+  acc.z += b.z;
+  acc.w += b.w;
+}
+
 // End of step t: the warps' partial sums are added in a fixed order (every
-// warp computes the same totals), then the Euler update of Eq. (1); warp 0
-// writes the trace, the last logit and the checkpoint.  Begins and ends with
-// a block barrier (the reduction buffer aliases the stage buffers).
+// warp computes the same totals), then the update of every sample.  Begins and
+// ends with a block barrier (the reduction buffer aliases the stage buffers).
 template <int D, int W, int K, bool TRACE>
 __device__ __forceinline__ void tile_finish_step(const TileArgs& a, int t, int64_t p0, const bool (&act)[K],
                                                  float (&x)[K][D], const float (&o)[D], bool expanded,
                                                  const u64 (&S)[K / 2], const u64 (&G)[K / 2][D], float4* red,
                                                  int warp, int lane) {
-  constexpr int P = K / 2;
   constexpr int kTile = 32 * K;
-  const int64_t N = a.N;
-  const float gamma = a.gamma, bias = a.bias, eta = a.eta;
-  const int T = a.T;
-  const float gl2e = gamma * kLog2e;
   __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
-#pragma unroll
-  for (int i = 0; i < P; ++i) {
-    float s0, s1, g0[D], g1[D];
-    upk(S[i], s0, s1);
-#pragma unroll
-    for (int j = 0; j < D; ++j) upk(G[i][j], g0[j], g1[j]);
-    red[warp * kTile + (2 * i) * 32 + lane] = make_float4(s0, g0[0], g0[1], D == 3 ? g0[D - 1] : 0.0f);
-    red[warp * kTile + (2 * i + 1) * 32 + lane] = make_float4(s1, g1[0], g1[1], D == 3 ? g1[D - 1] : 0.0f);
-  }
+  tile_put_sums<D, K>(S, G, red + warp * kTile, lane);
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     float4 acc = red[k * 32 + lane];
 #pragma unroll
-    for (int w = 1; w < W; ++w) {
-      float4 b = red[w * kTile + k * 32 + lane];
-      acc.x += b.x;
-      acc.y += b.y;
-      acc.z += b.z;
-      acc.w += b.w;
-    }
-    const float Ssum = acc.x, Gs[3] = {acc.y, acc.z, acc.w};
-    float shat, ghat[D];
-    if (expanded) {
-      float u[D], u2 = 0.0f;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        u[j] = x[k][j] - o[j];
-        u2 = fmaf(u[j], u[j], u2);
-      }
-      const float f = ex2_approx(-gl2e * u2);
-      shat = f * Ssum;
-#pragma unroll
-      for (int j = 0; j < D; ++j) ghat[j] = f * fmaf(u[j], Ssum, -Gs[j]);
-    } else {
-      shat = Ssum;
-#pragma unroll
-      for (int j = 0; j < D; ++j) ghat[j] = Gs[j];
-    }
-    float d1, d2;
-    sigmoid_d12(shat + bias, d1, d2);
-    const float c = -eta * d1;
-    const int64_t p = p0 + k * 32 + lane;
-    const bool own = act[k] && warp == 0;
-    const bool last_out = t == T - 1 && (a.s_out != nullptr || a.g_out != nullptr);
-    const int64_t n = (own && (TRACE || last_out)) ? (int64_t)a.perm[p] - a.perm_base : 0;
-    if (own && a.s_out != nullptr && t == T - 1) a.s_out[n] = shat + bias;
-    if (own && a.g_out != nullptr && t == T - 1)
-#pragma unroll
-      for (int j = 0; j < D; ++j) a.g_out[n * D + j] = d1 * (-2.0f * gamma * ghat[j]);
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      const float inc = __fmul_rn(c, -2.0f * gamma * ghat[j]);
-      if (TRACE && act[k] && warp == 0) {
-        a.traj[((int64_t)t * N + n) * D + j] = x[k][j];
-        a.steps[((int64_t)t * N + n) * D + j] = inc;
-      }
-      x[k][j] = __fadd_rn(x[k][j], inc);
-    }
+    for (int w = 1; w < W; ++w) add4(acc, red[w * kTile + k * 32 + lane]);
+    tile_update<D, K, TRACE>(a, t, p0, act, x, o, expanded, acc, k, warp == 0, lane);
   }
   __syncthreads();   // every warp has read the reduction buffer before the next step rebuilds the stages
-  if (a.ckpt != nullptr && (t + 1) % a.kck == 0 && warp == 0) {
-    float* dst = a.ckpt + (int64_t)((t + 1) / a.kck - 1) * N * D;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (act[k]) {
-        const int64_t n = (int64_t)a.perm[p0 + k * 32 + lane] - a.perm_base;
-#pragma unroll
-        for (int j = 0; j < D; ++j) dst[n * D + j] = x[k][j];
-      }
-  }
+  if (warp == 0) tile_checkpoint<D, K>(a, t, p0, act, x, lane);
 }
 
 // Writes x_T (and the trace's last state) of the tile's samples.
@@ -528,26 +643,84 @@ __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t p0, const 
   __syncthreads();   // the next tile of this block reuses the shared memory
 }
 
+// The sums S, G over the near groups of one walk, double-buffered through the
+// warp's two stages.  ORIGIN: see fast_tile.
+template <int D, int P, bool ORIGIN>
+__device__ __forceinline__ void near_sweep(const float4* __restrict__ tab, int64_t M, NearWalk walk, bool expanded,
+                                           const float (&o)[D], float gl2e, float4* wraw, u64* wbuf, int lane,
+                                           const u64 (&U)[P][D], u64 (&S)[P], u64 (&G)[P][D]) {
+  constexpr int RP = FastRec<D>::kPairs;
+  int g = walk.next();
+  if (g < 0) return;
+  u64* cur = wbuf;
+  u64* nxt = wbuf + (size_t)kWarpStage * RP;
+  stage_prefetch<D>(tab, M, (int64_t)g * kWarpStage, wraw, lane);
+  if (ORIGIN && !expanded)
+    stage_build_origin<D>(M, (int64_t)g * kWarpStage, o, gl2e, wraw, cur, lane);
+  else
+    stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, cur, lane);
+  __syncwarp();
+  do {
+    g = walk.next();
+    const int64_t mn = (int64_t)g * kWarpStage;
+    if (g >= 0) stage_prefetch<D>(tab, M, mn, wraw, lane);
+    if (ORIGIN && !expanded) {
+      stage_accumulate_origin<D, P>(cur, U, S, G);
+      if (g >= 0) stage_build_origin<D>(M, mn, o, gl2e, wraw, nxt, lane);
+    } else {
+      stage_accumulate<D, P>(cur, expanded, gl2e, U, S, G);
+      if (g >= 0) stage_build<D>(M, mn, expanded, o, gl2e, wraw, nxt, lane);
+    }
+    __syncwarp();
+    u64* const swap = cur;
+    cur = nxt;
+    nxt = swap;
+  } while (g >= 0);
+}
+
+// A tile's near groups are dealt out to kLeaves<W, K> partial sums, the totals
+// adding them in order.  Tiles of 320 samples have one per warp.  128-sample
+// tiles have 16 whatever the number of warps, so that a launch of few tiles
+// may spread a tile over a cluster of 2 or 4 blocks (CS) with the same result
+// bit for bit as one block of 4 warps that takes 4 leaves each.
+template <int W, int K>
+__host__ __device__ constexpr int tile_leaves() { return K == 4 ? 16 : W; }
+
+template <int D, int W, int K, int CS = 1>
+__host__ __device__ constexpr size_t tile_leaf_bytes() {
+  return tile_leaves<W, K>() == W ? 0
+                                  : (size_t)tile_leaves<W, K>() / CS * (CS > 1 ? 2 : 1) * (32 * K) * sizeof(float4);
+}
+// + near_bytes(M) at the end
+template <int D, int W, int K, int CS = 1>
+__host__ __device__ constexpr size_t tile_smem_bytes() {
+  return fast_smem_bytes<D, W, K>() + tile_leaf_bytes<D, W, K, CS>() +
+         (tile_leaves<W, K>() == W ? 0 : (size_t)32 * K * D * sizeof(float));
+}
+
 // ORIGIN: tiles too wide for the expanded form take the direct form about the
 // tile centre (stage_build_origin) instead of the one about 0.  The
 // single-field launch keeps the latter: there nearly every tile is expanded,
 // and the kernel compiled with both forms ran 6 % slower on such tiles.
-template <int D, int W, int K, bool TRACE, bool ORIGIN = false>
-__device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t p_end, unsigned char* smem) {
+// CS > 1: the tile is shared by the blocks of a cluster, this one of rank
+// crank; the launch is not persistent.
+template <int D, int W, int K, bool TRACE, bool ORIGIN = false, int CS = 1>
+__device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t p_end, unsigned char* smem,
+                                          int crank = 0) {
   constexpr int RP = FastRec<D>::kPairs;
   constexpr int P = K / 2;
   constexpr int KT = FastRec<D>::kTab;
+  constexpr int L = tile_leaves<W, K>(), WT = W * CS, kTile = 32 * K;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // each warp owns a contiguous slice of the centres and its own stage buffers
+  // each warp has its own stage buffers
   u64* wbuf = reinterpret_cast<u64*>(smem) + (size_t)warp * 2 * kWarpStage * RP;
   float4* red = reinterpret_cast<float4*>(smem);   // aliases the stage buffers after a step's last stage
   float4* wraw = reinterpret_cast<float4*>(smem + fast_region0_bytes<D, W, K>()) + (size_t)warp * kWarpStage * KT;
-  const float4* __restrict__ tab = a.tab;
-  const int64_t M = a.M;
+  float4* leaves = reinterpret_cast<float4*>(smem + fast_smem_bytes<D, W, K>());
+  float* xs = reinterpret_cast<float*>(smem + fast_smem_bytes<D, W, K>() + tile_leaf_bytes<D, W, K, CS>());
+  uint32_t* words = reinterpret_cast<uint32_t*>(smem + tile_smem_bytes<D, W, K, CS>());
   const float gl2e = a.gamma * kLog2e;
-  const int64_t Mw = ((M + W - 1) / W + kWarpStage - 1) / kWarpStage * kWarpStage;   // slice length
-  const int64_t mbase = (int64_t)warp * Mw;
-  const int nstage = (int)(Mw / kWarpStage);
+  const bool writer = warp == 0 && crank == 0;
 
   float x[K][D];
   bool act[K];
@@ -556,79 +729,89 @@ __device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t
   for (int t = 0; t < a.T; ++t) {
     float lo[D], hi[D], o[D];
     const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
+    near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
+    if (ORIGIN && !expanded)
+#pragma unroll
+      for (int j = 0; j < D; ++j) {   // the box's centre; 0 when the box is not finite
+        const float c = 0.5f * (lo[j] + hi[j]);
+        o[j] = c - c == 0.0f ? c : 0.0f;
+      }
+    const float us = !ORIGIN || expanded ? 1.0f : sqrtf(gl2e);
     u64 U[P][D], S[P], G[P][D];
-    if constexpr (ORIGIN) {
-      if (!expanded)
 #pragma unroll
-        for (int j = 0; j < D; ++j) {   // the box's centre; 0 when the box is not finite
-          const float c = 0.5f * (lo[j] + hi[j]);
-          o[j] = c - c == 0.0f ? c : 0.0f;
-        }
-      const float us = expanded ? 1.0f : sqrtf(gl2e);
+    for (int i = 0; i < P; ++i) {
 #pragma unroll
-      for (int i = 0; i < P; ++i) {
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          U[i][j] = pk(us * (x[2 * i][j] - o[j]), us * (x[2 * i + 1][j] - o[j]));
-          G[i][j] = 0ull;
-        }
-        S[i] = 0ull;
+      for (int j = 0; j < D; ++j) {
+        U[i][j] = ORIGIN ? pk(us * (x[2 * i][j] - o[j]), us * (x[2 * i + 1][j] - o[j]))
+                         : pk(x[2 * i][j] - o[j], x[2 * i + 1][j] - o[j]);
+        G[i][j] = 0ull;
       }
-      stage_prefetch<D>(tab, M, mbase, wraw, lane);
-      if (expanded)
-        stage_build<D>(M, mbase, true, o, gl2e, wraw, wbuf, lane);
-      else
-        stage_build_origin<D>(M, mbase, o, gl2e, wraw, wbuf, lane);
-      __syncwarp();
-      for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) stage_prefetch<D>(tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
-        u64* cur = wbuf + (size_t)(st & 1) * kWarpStage * RP;
-        u64* nxt = wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP;
-        const int64_t mn = mbase + (int64_t)(st + 1) * kWarpStage;
-        if (expanded) {
-          stage_accumulate<D, P>(cur, true, gl2e, U, S, G);
-          if (st + 1 < nstage) stage_build<D>(M, mn, true, o, gl2e, wraw, nxt, lane);
-        } else {
-          stage_accumulate_origin<D, P>(cur, U, S, G);
-          if (st + 1 < nstage) stage_build_origin<D>(M, mn, o, gl2e, wraw, nxt, lane);
-        }
-        __syncwarp();
-      }
-      if (!expanded) {
-        // to the direct form's moments: sum w phi (x - mu) = u S - G'
-        const u64 m1 = pk(-1.0f, -1.0f);
-#pragma unroll
-        for (int i = 0; i < P; ++i)
-#pragma unroll
-          for (int j = 0; j < D; ++j)
-            G[i][j] = fma2(pk(x[2 * i][j] - o[j], x[2 * i + 1][j] - o[j]), S[i], mul2(G[i][j], m1));
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < P; ++i) {
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          U[i][j] = pk(x[2 * i][j] - o[j], x[2 * i + 1][j] - o[j]);
-          G[i][j] = 0ull;
-        }
-        S[i] = 0ull;
-      }
-
-      stage_prefetch<D>(tab, M, mbase, wraw, lane);
-      stage_build<D>(M, mbase, expanded, o, gl2e, wraw, wbuf, lane);
-      __syncwarp();
-      for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) stage_prefetch<D>(tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
-        stage_accumulate<D, P>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, S, G);
-        if (st + 1 < nstage)
-          stage_build<D>(M, mbase + (int64_t)(st + 1) * kWarpStage, expanded, o, gl2e, wraw,
-                         wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP, lane);
-        __syncwarp();
-      }
+      S[i] = 0ull;
     }
-    tile_finish_step<D, W, K, TRACE>(a, t, p0, act, x, o, expanded, S, G, red, warp, lane);
+    // to the direct form's moments: sum w phi (x - mu) = u S - G'
+    auto from_origin = [&]() {
+      if (!ORIGIN || expanded) return;
+      const u64 m1 = pk(-1.0f, -1.0f);
+#pragma unroll
+      for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j)
+          G[i][j] = fma2(pk(x[2 * i][j] - o[j], x[2 * i + 1][j] - o[j]), S[i], mul2(G[i][j], m1));
+    };
+    __syncthreads();   // the near groups are marked
+    if constexpr (L == W) {
+      near_sweep<D, P, ORIGIN>(a.tab, a.M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U,
+                               S, G);
+      from_origin();
+      tile_finish_step<D, W, K, TRACE>(a, t, p0, act, x, o, expanded, S, G, red, warp, lane);
+    } else {
+      float4* buf = leaves + (CS > 1 ? (t & 1) * (L / CS) * kTile : 0);
+      for (int i = 0; i < L / WT; ++i) {
+        near_sweep<D, P, ORIGIN>(a.tab, a.M, NearWalk(words, a.ngroups, i * WT + crank * W + warp, L), expanded, o,
+                                 gl2e, wraw, wbuf, lane, U, S, G);
+        from_origin();
+        tile_put_sums<D, K>(S, G, buf + (i * W + warp) * kTile, lane);
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+          S[q] = 0ull;
+#pragma unroll
+          for (int j = 0; j < D; ++j) G[q][j] = 0ull;
+        }
+      }
+      // leaf l is slot (l / WT) W + (l % WT) % W of the block of rank (l % WT) / W
+      if (CS > 1) cluster_barrier(); else __syncthreads();
+      // warp w updates samples 32 w + lane (a quarter of the tile, so that a
+      // cluster's blocks read each other's leaves once) and shares them
+      static_assert(L == W || W == K, "a warp per 32 samples");
+      float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        const float4* src = buf + ((l / WT) * W + (l % WT) % W) * kTile + warp * 32 + lane;
+        const float4 v = CS > 1 ? cluster_load4(cluster_addr(src, (l % WT) / W)) : *src;
+        if (l == 0) acc = v; else add4(acc, v);
+      }
+      float xo[1][D];
+      bool ao[1];
+      ao[0] = p0 + warp * 32 + lane < p_end;
+#pragma unroll
+      for (int j = 0; j < D; ++j) xo[0][j] = x[0][j];
+#pragma unroll
+      for (int k = 1; k < K; ++k)
+#pragma unroll
+        for (int j = 0; j < D; ++j) xo[0][j] = warp == k ? x[k][j] : xo[0][j];
+      tile_update<D, 1, TRACE>(a, t, p0 + warp * 32, ao, xo, o, expanded, acc, 0, crank == 0, lane);
+      if (crank == 0) tile_checkpoint<D, 1>(a, t, p0 + warp * 32, ao, xo, lane);
+#pragma unroll
+      for (int j = 0; j < D; ++j) xs[j * kTile + warp * 32 + lane] = xo[0][j];
+      __syncthreads();   // the new samples are shared, the leaves read
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[k][j] = xs[j * kTile + k * 32 + lane];
+    }
   }
-  tile_store<D, K, TRACE>(a, p0, act, x, warp, lane);
+  if (CS > 1) cluster_barrier();      // no block leaves while another may read its leaves
+  tile_store<D, K, TRACE>(a, p0, act, x, writer ? 0 : 1, lane);
 }
 
 }  // namespace pdmp

@@ -145,13 +145,11 @@ __device__ __forceinline__ void inverse_tile(const TileArgs& a, float tol, int m
   const int64_t M = a.M;
   const float gl2e = a.gamma * kLog2e;
   const float m2g = -2.0f * a.gamma;
-  const int64_t Mw = ((M + W - 1) / W + kWarpStage - 1) / kWarpStage * kWarpStage;
-  const int64_t mbase = (int64_t)warp * Mw;
-  const int nstage = (int)(Mw / kWarpStage);
 
   float* zs = reinterpret_cast<float*>(smem + fast_smem_bytes<D, W, K>());   // kTile x D
   float* ds = zs + kTile * D;    // the corrections of the two steps undone before (warm start),
   float* ds2 = ds + kTile * D;   // kTile x D each
+  uint32_t* words = reinterpret_cast<uint32_t*>(ds2 + kTile * D);
   float y[K][D];
   bool act[K];
   tile_load<D, K>(a, p0, p_end, lane, y, act);
@@ -191,17 +189,10 @@ __device__ __forceinline__ void inverse_tile(const TileArgs& a, float tol, int m
         }
         S[i] = 0ull;
       }
-      stage_prefetch<D>(a.tab, M, mbase, wraw, lane);
-      stage_build<D>(M, mbase, expanded, o, gl2e, wraw, wbuf, lane);
-      __syncwarp();
-      for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) stage_prefetch<D>(a.tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
-        stage_accumulate<D, P>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, S, G);
-        if (st + 1 < nstage)
-          stage_build<D>(M, mbase + (int64_t)(st + 1) * kWarpStage, expanded, o, gl2e, wraw,
-                         wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP, lane);
-        __syncwarp();
-      }
+      near_mark<D, W, K>(a.box, a.ngroups, y, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
+      __syncthreads();   // the near groups are marked
+      near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
+                              G);
       __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
 #pragma unroll
       for (int i = 0; i < P; ++i) {
@@ -304,7 +295,8 @@ k_morph_inverse_fast(TileArgs a, float tol, int maxit, int32_t* __restrict__ ite
 template <int D, int K>
 static cudaError_t launch_inverse_shape(const TileArgs& a, float tol, int maxit, int32_t* iters,
                                         unsigned long long* work, cudaStream_t st) {
-  constexpr size_t smem = fast_smem_bytes<D, 4, K>() + 3 * (size_t)Shape<4, K>::kTile * D * sizeof(float);
+  const size_t smem =
+      fast_smem_bytes<D, 4, K>() + 3 * (size_t)Shape<4, K>::kTile * D * sizeof(float) + near_bytes(a.M);
   cudaError_t e =
       cudaFuncSetAttribute(k_morph_inverse_fast<D, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -317,20 +309,20 @@ template <int D>
 static cudaError_t launch_inverse_fast(const FieldArgs& fa, const float* z, int64_t N, int T, float eta, float tol,
                                       int maxit, float* y, int32_t* iters, unsigned long long* work, void* ws,
                                       cudaStream_t st) {
-  float4* tab = reinterpret_cast<float4*>(ws);
-  SortWs sw = sort_layout((char*)ws + rbf_fast_table_bytes(D, fa.M), D, N);
-  k_rbf_table<D><<<(unsigned)((fa.M + 255) / 256), 256, 0, st>>>(fa.centres, fa.w, fa.M, tab);
-  cudaError_t e = spatial_sort(D, z, N, sw, st);
+  RbfOrder ord;
+  cudaError_t e = rbf_order(D, fa.centres, fa.w, fa.M, z, N, ws, &ord, st);
   if (e != cudaSuccess) return e;
   TileArgs a{};
-  a.tab = tab;
+  a.tab = ord.tab;
+  a.box = ord.box;
+  a.ngroups = ord.ngroups;
   a.M = fa.M;
   a.gamma = fa.gamma;
   a.bias = fa.bias;
   a.eta = eta;
   a.T = T;
   a.x0 = z;
-  a.perm = sw.perm;
+  a.perm = ord.perm;
   a.perm_base = 0;
   a.N = N;
   a.xT = y;

@@ -12,8 +12,6 @@ cudaError_t morph_direct(int kind, int d, const FieldArgs& fa, const float* x0, 
                          float* xT, float* ckpt, int k, float* traj, float* steps, cudaStream_t st);
 // fast RBF path (d = 2, 3): spatially sorted tiles, expanded exponent, f32x2
 size_t morph_rbf_fast_workspace(int d, int64_t M, int64_t N);
-// bytes of the centre table at the start of that workspace (the sort's buffers follow)
-size_t rbf_fast_table_bytes(int d, int64_t M);
 size_t morph_rff_fast_workspace(int d, int64_t M);
 // RFF with both contractions on the tensor cores (d = 1 .. 7)
 size_t morph_rff_mma_workspace(int64_t M);
@@ -79,8 +77,10 @@ cudaError_t uniform_log_density(const float* y, int64_t N, int d, const double* 
                                 cudaStream_t st);
 
 int64_t vjp_blocks(int64_t N);
-// gw[m] = sum_b rows[b][m] (m < width - 1), *gbias = sum_b rows[b][width - 1], in block order
-cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st);
+// gw[perm[m]] = sum_b rows[b][m] (m < width - 1), *gbias = sum_b rows[b][width - 1], in block order
+// (perm NULL: the identity)
+cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st,
+                         const int32_t* perm = nullptr);
 // the tensor-core VJP for RFF fields (d <= 7, segments k <= kVjpMmaMaxSegment; ws: morph_rff_mma_workspace).
 // rows: nullptr, or vjp_rff_mma_blocks(N) x (M + 1) floats for the weight and bias gradient (gw, gbias)
 constexpr int kVjpMmaMaxSegment = 16;

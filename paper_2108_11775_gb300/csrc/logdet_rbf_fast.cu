@@ -173,15 +173,15 @@ __device__ __forceinline__ void ld_stage_accumulate(const u64* rec, bool expande
   }
 }
 
-// One sweep over the centres for the tile's samples x (every warp over its
-// slice of M, double-buffered stages); the per-warp sums S, G, H land in red
+// One sweep over the near groups of centres for the tile's samples x (words:
+// near_bytes; every warp over its own groups, double-buffered stages); the per-warp sums S, G, H land in red
 // ([W][NS][kTile] floats, aliasing the stages).  Returns whether the tile took
 // the expanded form, with its origin in o.  Ends with a block barrier after
 // the sums are written; the caller must pass another barrier before the next
 // sweep rebuilds the stages.
 template <int D, int K = kLdK<D>>
 __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][D], const bool (&act)[K],
-                                         float (&o)[D], unsigned char* smem, int warp, int lane) {
+                                         float (&o)[D], unsigned char* smem, uint32_t* words, int warp, int lane) {
   using L = LdRbf<D, K>;
   constexpr int W = L::kW, P = K / 2, RP = L::kPairs, NH = L::kH;
   constexpr int NS = L::kSums, kTile = L::kTile, KT = FastRec<D>::kTab;
@@ -190,12 +190,9 @@ __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][
   float4* wraw = reinterpret_cast<float4*>(smem + ld_rbf_region0<D, K>()) + (size_t)warp * kWarpStage * KT;
   const int64_t M = a.M;
   const float gl2e = a.gamma * kLog2e;
-  const int64_t Mw = ((M + W - 1) / W + kWarpStage - 1) / kWarpStage * kWarpStage;
-  const int64_t mbase = (int64_t)warp * Mw;
-  const int nstage = (int)(Mw / kWarpStage);
-
   float lo[D], hi[D];
   const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
+  near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
   u64 U[P][D], S[P], G[P][D], H[P][NH];
 #pragma unroll
   for (int i = 0; i < P; ++i) {
@@ -208,15 +205,21 @@ __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][
     for (int h = 0; h < NH; ++h) H[i][h] = 0ull;
     S[i] = 0ull;
   }
-  stage_prefetch<D>(a.tab, M, mbase, wraw, lane);
-  ld_stage_build<D>(M, mbase, expanded, o, gl2e, wraw, wbuf, lane);
+  __syncthreads();   // the near groups are marked
+  NearWalk walk(words, a.ngroups, warp, W);
+  int g = walk.next();
+  if (g >= 0) {
+    stage_prefetch<D>(a.tab, M, (int64_t)g * kWarpStage, wraw, lane);
+    ld_stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
+  }
   __syncwarp();
-  for (int st = 0; st < nstage; ++st) {
-    if (st + 1 < nstage) stage_prefetch<D>(a.tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
-    ld_stage_accumulate<D, P>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, S, G, H);
-    if (st + 1 < nstage)
-      ld_stage_build<D>(M, mbase + (int64_t)(st + 1) * kWarpStage, expanded, o, gl2e, wraw,
-                        wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP, lane);
+  for (int st = 0; g >= 0; st ^= 1) {
+    g = walk.next();
+    if (g >= 0) stage_prefetch<D>(a.tab, M, (int64_t)g * kWarpStage, wraw, lane);
+    ld_stage_accumulate<D, P>(wbuf + (size_t)st * kWarpStage * RP, expanded, gl2e, U, S, G, H);
+    if (g >= 0)
+      ld_stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, wbuf + (size_t)(st ^ 1) * kWarpStage * RP,
+                        lane);
     __syncwarp();
   }
   __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
@@ -321,6 +324,7 @@ k_logdet_rbf_fast(TileArgs a, float* __restrict__ logdet) {
   const float* red = reinterpret_cast<const float*>(smem);
   const int64_t p0 = (int64_t)blockIdx.x * kTile;
   const float eta = a.eta;
+  uint32_t* words = reinterpret_cast<uint32_t*>(smem + ld_rbf_smem<D>());
 
   float x[K][D];
   bool act[K];
@@ -335,7 +339,7 @@ k_logdet_rbf_fast(TileArgs a, float* __restrict__ logdet) {
 
   for (int t = 0; t < a.T; ++t) {
     float o[D];
-    const bool expanded = ld_sweep<D>(a, x, act, o, smem, warp, lane);
+    const bool expanded = ld_sweep<D>(a, x, act, o, smem, words, warp, lane);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       float shat, gs[D], hs[D][D];
@@ -391,6 +395,7 @@ k_log_density_rbf_fast(TileArgs a, float tol, int maxit, float* __restrict__ log
   float* zs = reinterpret_cast<float*>(smem + ld_rbf_smem<D, K>());   // kTile x D: the step's target z
   float* ds = zs + kTile * D;    // the corrections of the two steps undone before, kTile x D each
   float* ds2 = ds + kTile * D;
+  uint32_t* words = reinterpret_cast<uint32_t*>(ds2 + kTile * D);
 
   float y[K][D];
   bool act[K];
@@ -428,7 +433,7 @@ k_log_density_rbf_fast(TileArgs a, float tol, int maxit, float* __restrict__ log
     bool moving = true;
     while (moving && it < maxit) {
       float o[D];
-      const bool expanded = ld_sweep<D, K>(a, y, act, o, smem, warp, lane);
+      const bool expanded = ld_sweep<D, K>(a, y, act, o, smem, words, warp, lane);
       bool mv = false;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
@@ -493,24 +498,24 @@ k_log_density_rbf_fast(TileArgs a, float tol, int maxit, float* __restrict__ log
 template <int D>
 static cudaError_t launch_logdet_rbf_fast(const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, float* ld,
                                           float* xT, void* ws, cudaStream_t st) {
-  float4* tab = reinterpret_cast<float4*>(ws);
-  SortWs sw = sort_layout((char*)ws + rbf_fast_table_bytes(D, fa.M), D, N);
-  k_rbf_table<D><<<(unsigned)((fa.M + 255) / 256), 256, 0, st>>>(fa.centres, fa.w, fa.M, tab);
-  cudaError_t e = spatial_sort(D, x0, N, sw, st);
+  RbfOrder ord;
+  cudaError_t e = rbf_order(D, fa.centres, fa.w, fa.M, x0, N, ws, &ord, st);
   if (e != cudaSuccess) return e;
   TileArgs a{};
-  a.tab = tab;
+  a.tab = ord.tab;
+  a.box = ord.box;
+  a.ngroups = ord.ngroups;
   a.M = fa.M;
   a.gamma = fa.gamma;
   a.bias = fa.bias;
   a.eta = eta;
   a.T = T;
   a.x0 = x0;
-  a.perm = sw.perm;
+  a.perm = ord.perm;
   a.perm_base = 0;
   a.N = N;
   a.xT = xT;
-  constexpr size_t smem = ld_rbf_smem<D>();
+  const size_t smem = ld_rbf_smem<D>() + near_bytes(fa.M);
   e = cudaFuncSetAttribute(k_logdet_rbf_fast<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((N + LdRbf<D>::kTile - 1) / LdRbf<D>::kTile);
@@ -521,7 +526,8 @@ static cudaError_t launch_logdet_rbf_fast(const FieldArgs& fa, const float* x0, 
 template <int D, int K>
 static cudaError_t launch_log_density_shape(const TileArgs& a, float tol, int maxit, float* ld, int32_t* iters,
                                             unsigned long long* work, cudaStream_t st) {
-  constexpr size_t smem = ld_rbf_smem<D, K>() + 3 * (size_t)LdRbf<D, K>::kTile * D * sizeof(float);
+  const size_t smem =
+      ld_rbf_smem<D, K>() + 3 * (size_t)LdRbf<D, K>::kTile * D * sizeof(float) + near_bytes(a.M);
   cudaError_t e =
       cudaFuncSetAttribute(k_log_density_rbf_fast<D, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -534,20 +540,20 @@ template <int D>
 static cudaError_t launch_log_density_rbf_fast(const FieldArgs& fa, const float* z, int64_t N, int T, float eta,
                                                float tol, int maxit, float* y, float* ld, int32_t* iters,
                                                unsigned long long* work, void* ws, cudaStream_t st) {
-  float4* tab = reinterpret_cast<float4*>(ws);
-  SortWs sw = sort_layout((char*)ws + rbf_fast_table_bytes(D, fa.M), D, N);
-  k_rbf_table<D><<<(unsigned)((fa.M + 255) / 256), 256, 0, st>>>(fa.centres, fa.w, fa.M, tab);
-  cudaError_t e = spatial_sort(D, z, N, sw, st);
+  RbfOrder ord;
+  cudaError_t e = rbf_order(D, fa.centres, fa.w, fa.M, z, N, ws, &ord, st);
   if (e != cudaSuccess) return e;
   TileArgs a{};
-  a.tab = tab;
+  a.tab = ord.tab;
+  a.box = ord.box;
+  a.ngroups = ord.ngroups;
   a.M = fa.M;
   a.gamma = fa.gamma;
   a.bias = fa.bias;
   a.eta = eta;
   a.T = T;
   a.x0 = z;
-  a.perm = sw.perm;
+  a.perm = ord.perm;
   a.perm_base = 0;
   a.N = N;
   a.xT = y;

@@ -21,19 +21,20 @@
 // all 320 (10 per lane, five f32x2 pairs) and sums over its own contiguous
 // quarter of the centres; the four partial sums are added in a fixed order
 // once per step.  Launches too small to fill the GPU take 128-sample tiles
-// (below).
+// (below).  A sweep visits only the groups of centres that are not exactly
+// zero on the tile (fast_tile.cuh, rbf_order.cu).
 #include "fast_tile.cuh"
 #include "kernels.cuh"
 #include "sort.cuh"
 
 namespace pdmp {
 
-template <int D, bool TRACE, int K>
+template <int D, bool TRACE, int K, int CS>
 __global__ void __launch_bounds__(Shape<4, K>::kThreads, Shape<4, K>::kMinBlocks)
 k_morph_rbf_fast(TileArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int64_t p0 = (int64_t)blockIdx.x * Shape<4, K>::kTile;
-  fast_tile<D, 4, K, TRACE>(a, p0, a.N, smem);
+  const int64_t p0 = (int64_t)(blockIdx.x / CS) * Shape<4, K>::kTile;
+  fast_tile<D, 4, K, TRACE, false, CS>(a, p0, a.N, smem, (int)(blockIdx.x % CS));
 }
 
 // Samples per lane.  A launch of fewer 320-sample tiles than fit on the GPU at
@@ -43,61 +44,79 @@ k_morph_rbf_fast(TileArgs a) {
 // 2^18 samples) the larger tiles are as fast or faster.
 constexpr int kSmallK = 4;
 
-static int fast_samples_per_lane(int64_t N) {
+static int num_sms() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                  cudaSuccess || sms < 1)
     sms = 152;
-  const int64_t tiles = (N + FastShape::kTile - 1) / FastShape::kTile;
-  return tiles < (int64_t)FastShape::kMinBlocks * sms ? kSmallK : FastShape::kK;
+  return sms;
 }
 
 // ------------------------------------------------------------------ host
-size_t rbf_fast_table_bytes(int d, int64_t M) {
-  return (((size_t)M * 16 * (d == 2 ? 1 : 2)) + 255) & ~size_t(255);
-}
+size_t morph_rbf_fast_workspace(int d, int64_t M, int64_t N) { return rbf_order_workspace(d, M, N); }
 
-size_t morph_rbf_fast_workspace(int d, int64_t M, int64_t N) {
-  return rbf_fast_table_bytes(d, M) + sort_workspace(d, N);
-}
-
-template <int D, int K>
-static cudaError_t launch_shape(const TileArgs& a, int64_t N, bool trace, cudaStream_t st) {
-  constexpr size_t smem = fast_smem_bytes<D, 4, K>();
-  const unsigned blocks = (unsigned)((N + Shape<4, K>::kTile - 1) / Shape<4, K>::kTile);
-  cudaError_t e;
-  if (trace) {
-    e = cudaFuncSetAttribute(k_morph_rbf_fast<D, true, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_morph_rbf_fast<D, true, K><<<blocks, Shape<4, K>::kThreads, smem, st>>>(a);
-  } else {
-    e = cudaFuncSetAttribute(k_morph_rbf_fast<D, false, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_morph_rbf_fast<D, false, K><<<blocks, Shape<4, K>::kThreads, smem, st>>>(a);
+template <int D, bool TRACE, int K, int CS>
+static cudaError_t launch_shape(const TileArgs& a, int64_t N, cudaStream_t st) {
+  const size_t smem = tile_smem_bytes<D, 4, K, CS>() + near_bytes(a.M);
+  const unsigned blocks = (unsigned)((N + Shape<4, K>::kTile - 1) / Shape<4, K>::kTile) * CS;
+  auto fn = k_morph_rbf_fast<D, TRACE, K, CS>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  if (CS == 1) {
+    fn<<<blocks, Shape<4, K>::kThreads, smem, st>>>(a);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(blocks);
+  c.blockDim = dim3(Shape<4, K>::kThreads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, fn, a);
+}
+
+// 128-sample tiles go to a cluster of 4 blocks while there are fewer tiles than
+// SMs, to 2 while there are fewer than two per SM: one block of four warps an
+// SM leaves each scheduler a single warp.  Measured (2-D, T = 10): 4096 samples
+// and 1024 centres 62 us on clusters of 4; the call with its order 73 us
+// against 131 us of one block a tile and the eight-launch sort.
+template <int D, bool TRACE>
+static cudaError_t launch_tiles(const TileArgs& a, int64_t N, cudaStream_t st) {
+  const int64_t sms = num_sms();
+  const int64_t tiles = (N + FastShape::kTile - 1) / FastShape::kTile;
+  if (tiles >= FastShape::kMinBlocks * sms) return launch_shape<D, TRACE, FastShape::kK, 1>(a, N, st);
+  const int64_t small = (N + Shape<4, kSmallK>::kTile - 1) / Shape<4, kSmallK>::kTile;
+  if (small <= sms) return launch_shape<D, TRACE, kSmallK, 4>(a, N, st);
+  if (small <= 2 * sms) return launch_shape<D, TRACE, kSmallK, 2>(a, N, st);
+  return launch_shape<D, TRACE, kSmallK, 1>(a, N, st);
 }
 
 template <int D>
 static cudaError_t launch_fast(const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, float* xT,
                                float* ckpt, int k, float* traj, float* steps, void* ws, cudaStream_t st,
                                float* s_out, float* g_out = nullptr) {
-  float4* tab = reinterpret_cast<float4*>(ws);
-  SortWs sw = sort_layout((char*)ws + rbf_fast_table_bytes(D, fa.M), D, N);
-  cudaError_t e = spatial_sort(D, x0, N, sw, st);
+  RbfOrder ord;
+  cudaError_t e = rbf_order(D, fa.centres, fa.w, fa.M, x0, N, ws, &ord, st);
   if (e != cudaSuccess) return e;
   if (morph_rbf_tc05_eligible(D, N))
-    return morph_rbf_tc05(D, fa, x0, sw.perm, N, T, eta, xT, ckpt, k, traj, steps, s_out, g_out, st);
-  k_rbf_table<D><<<(unsigned)((fa.M + 255) / 256), 256, 0, st>>>(fa.centres, fa.w, fa.M, tab);
-  TileArgs a;
-  a.tab = tab;
+    return morph_rbf_tc05(D, fa, x0, ord.perm, N, T, eta, xT, ckpt, k, traj, steps, s_out, g_out, st);
+  TileArgs a{};
+  a.tab = ord.tab;
+  a.box = ord.box;
+  a.ngroups = ord.ngroups;
   a.M = fa.M;
   a.gamma = fa.gamma;
   a.bias = fa.bias;
   a.eta = eta;
   a.T = T;
   a.x0 = x0;
-  a.perm = sw.perm;
+  a.perm = ord.perm;
   a.perm_base = 0;
   a.N = N;
   a.xT = xT;
@@ -107,8 +126,7 @@ static cudaError_t launch_fast(const FieldArgs& fa, const float* x0, int64_t N, 
   a.steps = steps;
   a.s_out = s_out;
   a.g_out = g_out;
-  if (fast_samples_per_lane(N) == kSmallK) return launch_shape<D, kSmallK>(a, N, traj != nullptr, st);
-  return launch_shape<D, FastShape::kK>(a, N, traj != nullptr, st);
+  return traj != nullptr ? launch_tiles<D, true>(a, N, st) : launch_tiles<D, false>(a, N, st);
 }
 
 cudaError_t morph_rbf_fast(int d, const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, float* xT,

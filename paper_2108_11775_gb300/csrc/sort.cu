@@ -15,6 +15,7 @@
 // and so can the rounding of the results (within the kernels' accuracy: the
 // tile a sample falls in changes only the rounding of its arithmetic).
 #include "kernels.cuh"
+#include "order.cuh"
 #include "sort.cuh"
 
 namespace pdmp {
@@ -60,35 +61,6 @@ __global__ void k_cell_keys(const float* __restrict__ x, int64_t N, const uint32
 }
 
 // exclusive scan of counts[0..C) into offs, in chunks of kScanChunk
-
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* sh, uint32_t& total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  if (lane == 31) sh[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0u;
-    uint32_t wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += t;
-    }
-    sh[lane] = wi - w;
-    if (lane == 31) sh[32] = wi;
-  }
-  __syncthreads();
-  uint32_t r = inc - v + sh[warp];
-  total = sh[32];
-  __syncthreads();
-  return r;
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_scan_chunks(const uint32_t* __restrict__ counts, int64_t C,
                                                               uint32_t* __restrict__ offs,
                                                               uint32_t* __restrict__ chunk_tot) {

@@ -75,10 +75,17 @@ __device__ __forceinline__ uint32_t hilbert_key(uint32_t (&c)[n], int bits) {
 
 // cell index in [0, cells) of v along one axis of the box [lo, hi]; NaN and
 // values below lo give 0, values at or above hi give cells - 1
-__device__ __forceinline__ uint32_t cell_coord(float v, float lo, float hi, float cells) {
+// (scale: cell_scale(lo, hi, cells), negative when the box has no extent)
+__device__ __forceinline__ float cell_scale(float lo, float hi, float cells) {
   const float span = hi - lo;
-  const float q = span > 0.0f ? (v - lo) * (cells / span) : 0.0f;
+  return span > 0.0f ? cells / span : -1.0f;
+}
+__device__ __forceinline__ uint32_t cell_at(float v, float lo, float scale, float cells) {
+  const float q = scale >= 0.0f ? (v - lo) * scale : 0.0f;
   return (q >= 0.0f) ? (uint32_t)fminf(q, cells - 1.0f) : 0u;
+}
+__device__ __forceinline__ uint32_t cell_coord(float v, float lo, float hi, float cells) {
+  return cell_at(v, lo, cell_scale(lo, hi, cells), cells);
 }
 
 struct SortWs {

@@ -250,21 +250,23 @@ k_morph_vjp(FieldArgs fa, const float* __restrict__ x0, int64_t N, int T, float 
 }
 
 // sums the per-block rows in block order: out[m] = sum_b rows[b][m], m <= M
+// (perm: NULL, or the feature of each row position)
 __global__ void k_sum_rows(const float* __restrict__ rows, int64_t nrows, int64_t width, float* __restrict__ gw,
-                           float* __restrict__ gbias) {
+                           float* __restrict__ gbias, const int32_t* __restrict__ perm) {
   int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= width) return;
   float acc = 0.0f;
   for (int64_t b = 0; b < nrows; ++b) acc += rows[b * width + m];
   if (m + 1 < width) {
-    if (gw) gw[m] = acc;
+    if (gw) gw[perm ? perm[m] : m] = acc;
   } else if (gbias) {
     *gbias = acc;
   }
 }
 
-cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st) {
-  k_sum_rows<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(rows, nrows, width, gw, gbias);
+cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st,
+                         const int32_t* perm) {
+  k_sum_rows<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(rows, nrows, width, gw, gbias, perm);
   return cudaGetLastError();
 }
 

@@ -75,23 +75,31 @@ struct GwTerms {
   }
 };
 
-// The weight-gradient sweep of one warp over its slice [m_lo, m_hi) of the
-// features (sm: the tile's sample terms); adds each feature's sum to row[m].
+// The weight-gradient sweep of one warp over its near groups of features (sm:
+// the tile's sample terms), a feature a lane and kGwFeatures groups at a time;
+// adds each feature's sum to row (in table order).
 template <int D, int kTile>
-__device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int64_t m_lo, int64_t m_hi,
+__device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int64_t M, NearWalk walk,
                                             bool expanded, const float* o, float gl2e, const float* sm,
                                             float* __restrict__ row, int lane) {
   constexpr int TP = GwTerms<D>::kPairs;
   constexpr int KT = FastRec<D>::kTab;
   constexpr int F = kGwFeatures;
-  for (int64_t m0 = m_lo; m0 < m_hi; m0 += 32 * F) {
+  for (;;) {
+    int64_t mf[F];
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+      const int g = walk.next();
+      mf[f] = g < 0 ? M : (int64_t)g * kGroup + lane;
+    }
+    if (mf[0] >= M && __all_sync(0xffffffffu, mf[0] >= M)) break;
     u64 cst[F], bm[F][D], A[F], Q[F][D];
     float c[F][D];
     bool ok[F];
 #pragma unroll
     for (int f = 0; f < F; ++f) {
-      const int64_t m = m0 + f * 32 + lane;
-      ok[f] = m < m_hi;
+      const int64_t m = mf[f];
+      ok[f] = m < M;
       float mu[D];
       if (ok[f]) {
         const float4 t0 = tab[KT * m];
@@ -173,7 +181,7 @@ __device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int6
         upk(Q[f][j], lo, hi);
         v = fmaf(c[f][j], lo + hi, v);
       }
-      row[m0 + f * 32 + lane] += v;
+      row[mf[f]] += v;
     }
   }
 }
@@ -322,14 +330,15 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
   const int64_t p0 = (int64_t)blockIdx.x * kTile;
   const int64_t N = a.N, M = a.M;
   const float gamma = a.gamma, gl2e = gamma * kLog2e, eta = a.eta;
-  const int64_t Mw = ((M + W - 1) / W + kWarpStage - 1) / kWarpStage * kWarpStage;
-  const int64_t mbase = (int64_t)warp * Mw;
-  const int nstage = (int)(Mw / kWarpStage);
-  // weight gradient: this block's row of rows[blocks][M + 1] and the sample terms after the segment
+  // with the weight gradient a ragged tile visits every group: its empty slots sit at 0, where the expanded
+  // sums can overflow, and what they then add to the row has to stay what it is without far groups
+  const bool whole = GW && p0 + kTile > N;
+  // weight gradient: this block's row of rows[blocks][M + 1] (features in table order) and the sample terms after the segment
   float* row = GW ? rows + (int64_t)blockIdx.x * (M + 1) : nullptr;
   // the forward's S, G (cross-warp totals) at the segment's states: [kseg][1 + D][kTile]
   float* sgc = seg + (size_t)kseg * kTile * D;
   float* sm_gw = sgc + (use_cache ? (size_t)kseg * (1 + D) * kTile : 0);   // [kTile / 2][2D + 2] packed pairs
+  uint32_t* words = reinterpret_cast<uint32_t*>(sm_gw + (GW ? (2 * D + 2) * kTile : 0));
   if (GW)
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
   float gb = 0.0f;   // warp 0: the bias term of this lane's samples
@@ -376,17 +385,10 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         }
         S[q] = 0ull;
       }
-      stage_prefetch<D>(a.tab, M, mbase, wraw, lane);
-      stage_build<D>(M, mbase, expanded, o, gl2e, wraw, wbuf, lane);
-      __syncwarp();
-      for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) stage_prefetch<D>(a.tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
-        stage_accumulate<D, P>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, S, G);
-        if (st + 1 < nstage)
-          stage_build<D>(M, mbase + (int64_t)(st + 1) * kWarpStage, expanded, o, gl2e, wraw,
-                         wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP, lane);
-        __syncwarp();
-      }
+      near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, whole, words, warp, lane);
+      __syncthreads();   // the near groups are marked
+      near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
+                              G);
       tile_finish_step<D, W, K, false>(a, 0, p0, act, x, o, expanded, S, G, reinterpret_cast<float4*>(red), warp,
                                        lane);
       if (use_cache && i >= pre) {
@@ -436,18 +438,27 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         for (int h = 0; h < NH; ++h) H[q][h] = 0ull;
         S[q] = 0ull;
       }
-      stage_prefetch<D>(a.tab, M, mbase, wraw, lane);
-      vj_stage_build<D>(M, mbase, expanded, o, gl2e, wraw, wbuf, lane);
+      // with the weight gradient, whose sums take phi without its weight, near for those too
+      near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, GW, whole, words, warp, lane);
+      __syncthreads();   // the near groups are marked
+      NearWalk walk(words, a.ngroups, warp, W);
+      int gi = walk.next();
+      if (gi >= 0) {
+        stage_prefetch<D>(a.tab, M, (int64_t)gi * kWarpStage, wraw, lane);
+        vj_stage_build<D>(M, (int64_t)gi * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
+      }
       __syncwarp();
-      for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) stage_prefetch<D>(a.tab, M, mbase + (int64_t)(st + 1) * kWarpStage, wraw, lane);
+      for (int st = 0; gi >= 0; st ^= 1) {
+        gi = walk.next();
+        const u64* cur = wbuf + (size_t)st * kWarpStage * RP;
+        if (gi >= 0) stage_prefetch<D>(a.tab, M, (int64_t)gi * kWarpStage, wraw, lane);
         if (have)
-          vj_stage_accumulate<D, P, false>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, V, S, G, H);
+          vj_stage_accumulate<D, P, false>(cur, expanded, gl2e, U, V, S, G, H);
         else
-          vj_stage_accumulate<D, P, true>(wbuf + (size_t)(st & 1) * kWarpStage * RP, expanded, gl2e, U, V, S, G, H);
-        if (st + 1 < nstage)
-          vj_stage_build<D>(M, mbase + (int64_t)(st + 1) * kWarpStage, expanded, o, gl2e, wraw,
-                            wbuf + (size_t)((st + 1) & 1) * kWarpStage * RP, lane);
+          vj_stage_accumulate<D, P, true>(cur, expanded, gl2e, U, V, S, G, H);
+        if (gi >= 0)
+          vj_stage_build<D>(M, (int64_t)gi * kWarpStage, expanded, o, gl2e, wraw,
+                            wbuf + (size_t)(st ^ 1) * kWarpStage * RP, lane);
         __syncwarp();
       }
       __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
@@ -554,8 +565,10 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         for (int j = 0; j < D; ++j) g[k][j] = g[k][j] - eta * fmaf(d1, hv[j], d2 * gd * gs[j]);
       }
       __syncthreads();   // every warp has read the reduction buffer before the next pass rebuilds the stages
-      if (GW)            // (and the sample terms are visible)
-        vj_gw_sweep<D, kTile>(a.tab, mbase, mbase + Mw < M ? mbase + Mw : M, expanded, o, gl2e, sm_gw, row, lane);
+      if (GW) {          // (and the sample terms are visible)
+        vj_gw_sweep<D, kTile>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, sm_gw, row, lane);
+        __syncthreads();   // every warp has walked the groups and read the terms before the next pass marks them
+      }
     }
   }
   if (GW && warp == 0) {
@@ -575,20 +588,20 @@ template <int D>
 static cudaError_t launch_vjp_rbf_fast(const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, int k,
                                        const float* ckpt, const float* gT, float* g0, float* rows, float* gw,
                                        float* gbias, void* ws, cudaStream_t st) {
-  float4* tab = reinterpret_cast<float4*>(ws);
-  SortWs sw = sort_layout((char*)ws + rbf_fast_table_bytes(D, fa.M), D, N);
-  k_rbf_table<D><<<(unsigned)((fa.M + 255) / 256), 256, 0, st>>>(fa.centres, fa.w, fa.M, tab);
-  cudaError_t e = spatial_sort(D, x0, N, sw, st);
+  RbfOrder ord;
+  cudaError_t e = rbf_order(D, fa.centres, fa.w, fa.M, x0, N, ws, &ord, st);
   if (e != cudaSuccess) return e;
   TileArgs a{};
-  a.tab = tab;
+  a.tab = ord.tab;
+  a.box = ord.box;
+  a.ngroups = ord.ngroups;
   a.M = fa.M;
   a.gamma = fa.gamma;
   a.bias = fa.bias;
   a.eta = eta;
   a.T = T;
   a.x0 = x0;
-  a.perm = sw.perm;
+  a.perm = ord.perm;
   a.perm_base = 0;
   a.N = N;
   a.kck = 1;
@@ -596,7 +609,8 @@ static cudaError_t launch_vjp_rbf_fast(const FieldArgs& fa, const float* x0, int
   const void* fn = want ? reinterpret_cast<const void*>(k_vjp_rbf_fast<D, true>)
                         : reinterpret_cast<const void*>(k_vjp_rbf_fast<D, false>);
   // cache the recompute's S and G when the extra shared memory keeps as many blocks on an SM
-  const size_t smem0 = vj_rbf_smem<D>(k, want, false), smem1 = vj_rbf_smem<D>(k, want, true);
+  const size_t nb = near_bytes(fa.M);
+  const size_t smem0 = vj_rbf_smem<D>(k, want, false) + nb, smem1 = vj_rbf_smem<D>(k, want, true) + nb;
   int b0 = 0, b1 = 0;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
   if (e != cudaSuccess) return e;
@@ -613,7 +627,7 @@ static cudaError_t launch_vjp_rbf_fast(const FieldArgs& fa, const float* x0, int
   k_vjp_rbf_fast<D, true><<<blocks, VjRbf<D>::kW * 32, smem, st>>>(a, k, ckpt, gT, g0, rows, use_cache);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return sum_vjp_rows(rows, (int64_t)blocks, fa.M + 1, gw, gbias, st);
+  return sum_vjp_rows(rows, (int64_t)blocks, fa.M + 1, gw, gbias, st, ord.cperm);
 }
 
 int64_t vjp_rbf_fast_blocks(int d, int64_t N) {
