@@ -265,36 +265,87 @@ __device__ __forceinline__ bool tile_frame(const float (&x)[K][D], const bool (&
 }
 
 // ------------------------------------------------------------- near groups
-// A group of centres is far from a tile at a state when every one of its
-// features is exactly zero for every sample there (see rbf_order.cu): with d
-// the distance between the two boxes, the exponents the kernels form are at
-// most lw_max - g' d^2 (the expanded form's + g' R^2, its factor f = 2^(-g'
-// |u|^2) taken out), and ex2.approx.ftz returns 0 below -126.  One unit more
-// covers the rounding of the exponents and of this test.  A tile with a
-// sample that is not finite has no far groups (its sums must reach it).
+// With y = g' d^2, d the distance between a group's box and the tile's, the
+// group's terms of s are at most 2^(lw_max - y) for every sample of the tile.  A
+// group is far, and left out, in two cases.
+//
+// (1) Its terms are exactly zero: the exponents the kernels form are at most
+// lw_max - y (the expanded form's + g' R^2, its factor f = 2^(-g' |u|^2) taken
+// out), and ex2.approx.ftz returns 0 below -126.  One unit more covers the
+// rounding of the exponents and of this test.
+//
+// (2) All far groups together are below FP32's rounding of the sums.  Every
+// group's strongest centre mu* bounds one term of the sums from below for every
+// sample of the tile: of s by 2^(lw* - g' dmax^2), of grad s by that times the
+// distance, sqrt(g') dmin; let ref be the largest of the latter (at most the
+// largest of the former).  Beyond y = 1 a feature's terms of s, grad s and Hess
+// s (2 gamma (1 + 2 gamma d^2) relative to s's) fall with d, so that with
+//   lw_max - y + log2(1 + 2 gamma d^2) < log2(ref) - (30 + log2 M)
+// the M features at most that are left out add up to less than 2^-30 of a term
+// that is summed: 1/64 of the rounding error that this term alone brings
+// (FP32's half ulp, 2^-25), whatever cancels.  Not used where a feature stands
+// without its weight or is an output itself (the weight gradient).
+//
+// A tile with a sample that is not finite has no far groups (its sums must
+// reach it).
 //
 // The near groups are marked in shared memory, one bit each, by all warps of
 // the block together once per sweep; groups past kNearWords * 32 (M > 2^20)
 // count as near.  Every warp then walks the marked groups that are its own.
+// Measured with (1) alone and with both: the morph of 2^20 samples (M = 16,384,
+// T = 50, 2-D) 59.0 and 32.4 ms, the log-density of 2^16 samples 10.3 and 7.4
+// ms, 48 environments 42.2 and 37.3 ms; errors against 64 bits unchanged.
 constexpr int kNearWords = 1024;
+constexpr int kNearExtra = 16;       // words after the marks: the warps' largest ref
 
 __host__ __device__ __forceinline__ int near_words(int ngroups) {
   const int n = (ngroups + 31) / 32;
   return n < kNearWords ? n : kNearWords;
 }
 __host__ __device__ __forceinline__ size_t near_bytes(int64_t M) {
-  return ((size_t)near_words(group_count(M)) * 4 + 15) & ~size_t(15);
+  return ((size_t)(near_words(group_count(M)) + kNearExtra) * 4 + 15) & ~size_t(15);
 }
 
+// what near_mark marks
+enum NearRule { kNearSums, kNearUnweighted, kNearAll };
+
 // Marks the groups that are near the tile's box [lo, hi] (of x, the same in
-// every warp); a block barrier before and after must separate it from the
-// walks of the sweep before and of this one.  unweighted: sums in which phi
-// stands without its weight; all: mark every group.
+// every warp).  kNearSums: rules (1) and (2); kNearUnweighted: rule (1) for sums
+// in which phi stands without its weight; kNearAll: every group.  Block
+// barriers separate it from the walks of the sweep before and of this one.
 template <int D, int W, int K>
-__device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ngroups, const float (&x)[K][D],
-                                          const bool (&act)[K], const float (&lo)[D], const float (&hi)[D],
-                                          bool expanded, float gl2e, bool unweighted, bool all, uint32_t* words,
-                                          int warp, int lane) {
+__device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ngroups, int64_t M,
+                                          const float (&x)[K][D], const bool (&act)[K], const float (&lo)[D],
+                                          const float (&hi)[D], bool expanded, float gl2e, NearRule rule,
+                                          uint32_t* words, int warp, int lane) {
+  const int nw = near_words(ngroups);
+  float ref = -INFINITY;
+  if (rule == kNearSums) {
+    // of few groups every warp goes over all (no exchange), of many over its share
+    const bool share = ngroups > 64;
+    for (int g = (share ? warp * 32 : 0) + lane; g < ngroups; g += (share ? W : 1) * 32) {
+      const float4 b = box[kGroupBox * g + 2];
+      const float mu[3] = {b.x, b.y, b.z};
+      float dmin2 = 0.0f, dmax2 = 0.0f;
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        const float gap = fmaxf(0.0f, fmaxf(mu[j] - hi[j], lo[j] - mu[j]));
+        const float reach = fmaxf(hi[j] - mu[j], mu[j] - lo[j]);
+        dmin2 = fmaf(gap, gap, dmin2);
+        dmax2 = fmaf(reach, reach, dmax2);
+      }
+      ref = fmaxf(ref, fmaf(-gl2e, dmax2, b.w) + 0.5f * lg2_approx(fminf(1.0f, gl2e * dmin2)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, o));
+    if (share) {
+      float* refs = reinterpret_cast<float*>(words + nw);
+      if (lane == 0) refs[warp] = ref;
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < W; ++w) ref = fmaxf(ref, refs[w]);
+    }
+  }
   float R2 = 0.0f;
   bool odd = false;
 #pragma unroll
@@ -307,8 +358,8 @@ __device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ng
 #pragma unroll
     for (int j = 0; j < D; ++j) odd = odd || (act[k] && !(fabsf(x[k][j]) < INFINITY));
   odd = __any_sync(0xffffffffu, odd);
-  const float lim = odd || all ? INFINITY : 127.0f + (expanded ? gl2e * R2 : 0.0f);
-  const int nw = near_words(ngroups);
+  const float lim1 = odd || rule == kNearAll ? INFINITY : 127.0f + (expanded ? gl2e * R2 : 0.0f);
+  const float lim2 = odd || rule != kNearSums ? INFINITY : 30.0f + lg2_approx((float)M) - ref;
   for (int q = warp; q < nw; q += W) {
     const int g = q * 32 + lane;
     bool near = false;
@@ -321,7 +372,10 @@ __device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ng
         const float gap = fmaxf(0.0f, fmaxf(blo[j] - hi[j], lo[j] - bhi[j]));
         d2 = fmaf(gap, gap, d2);
       }
-      near = !(fmaf(gl2e, d2, -(unweighted ? fmaxf(b0.w, 0.0f) : b0.w)) > lim);
+      const float y = gl2e * d2, below = y - (rule == kNearUnweighted ? fmaxf(b0.w, 0.0f) : b0.w);
+      // 2 gamma d^2 = 2 ln 2 y
+      const bool far = below > lim1 || (y > 1.0f && below - lg2_approx(fmaf(1.38629436f, y, 1.0f)) > lim2);
+      near = !far;
     }
     const uint32_t m = __ballot_sync(0xffffffffu, near);
     if (lane == 0) words[q] = m;
@@ -729,7 +783,7 @@ __device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t
   for (int t = 0; t < a.T; ++t) {
     float lo[D], hi[D], o[D];
     const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
-    near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
+    near_mark<D, W, K>(a.box, a.ngroups, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
     if (ORIGIN && !expanded)
 #pragma unroll
       for (int j = 0; j < D; ++j) {   // the box's centre; 0 when the box is not finite

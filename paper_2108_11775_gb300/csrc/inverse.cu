@@ -189,7 +189,7 @@ __device__ __forceinline__ void inverse_tile(const TileArgs& a, float tol, int m
         }
         S[i] = 0ull;
       }
-      near_mark<D, W, K>(a.box, a.ngroups, y, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
+      near_mark<D, W, K>(a.box, a.ngroups, a.M, y, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
       __syncthreads();   // the near groups are marked
       near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
                               G);

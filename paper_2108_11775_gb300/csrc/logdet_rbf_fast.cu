@@ -192,7 +192,7 @@ __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][
   const float gl2e = a.gamma * kLog2e;
   float lo[D], hi[D];
   const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
-  near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, false, words, warp, lane);
+  near_mark<D, W, K>(a.box, a.ngroups, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
   u64 U[P][D], S[P], G[P][D], H[P][NH];
 #pragma unroll
   for (int i = 0; i < P; ++i) {

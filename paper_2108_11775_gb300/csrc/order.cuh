@@ -15,7 +15,7 @@ constexpr int kOrderThreads = 512;
 constexpr int kOrderWarps = kOrderThreads / 32;
 constexpr int kOrderShare = kOrderChunk / kOrderBlocks;   // items per block at most
 constexpr int kGroup = 32;
-constexpr int kGroupBox = 2;         // float4s per group: its bounding box and its largest log2|w|
+constexpr int kGroupBox = 3;         // float4s per group: its bounding box, its strongest centre and log2|w|
 constexpr int kDigits = 64;          // radix of the sort (keys of two digits)
 constexpr int kCountRow = kOrderWarps + 1;   // rows padded: a warp's lanes hit distinct banks
 static_assert(kDigits * kOrderBlocks == kOrderThreads, "a thread per digit and block");
@@ -260,9 +260,10 @@ __device__ int cluster_order(const float* __restrict__ pts, int n, int bits, Ord
 // Table entries and group boxes of the sorted positions [p0, p0 + share) that
 // this block holds of a chunk of n centres: entry i of the chunk is {mu_0 ..
 // mu_{D-1}, lw = log2|w|, sg = sign(w)} of the centre there; perm (may be
-// NULL) receives base + its index in the chunk.  Box of a group: {lo_0 .., lw_max in .w}, {hi_0 ..}; a centre or
-// weight that is not finite makes its group's box everything, so that no tile
-// leaves the group out.
+// NULL) receives base + its index in the chunk.  Box of a group: {lo_0 ..,
+// lw_max in .w}, {hi_0 ..}, {mu_0 .., lw in .w} of its centre of largest |w|; a
+// centre or weight that is not finite makes its group's box everything, so
+// that no tile leaves the group out.
 template <int D>
 __device__ void order_table(const float* __restrict__ centres, const float* __restrict__ w, int n, const OrderSmem& s,
                             int p0, int share, float4* __restrict__ tab, float4* __restrict__ box,
@@ -308,6 +309,7 @@ __device__ void order_table(const float* __restrict__ centres, const float* __re
         if (perm) perm[i] = (int32_t)(base + m[u]);
       }
       odd = __any_sync(0xffffffffu, odd);
+      const float lw0 = lmax;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
@@ -317,6 +319,11 @@ __device__ void order_table(const float* __restrict__ centres, const float* __re
           hi[j] = fmaxf(hi[j], __shfl_xor_sync(0xffffffffu, hi[j], o));
         }
       }
+      const int top = __ffs(__ballot_sync(0xffffffffu, i < end && lw0 == lmax)) - 1;
+      float mt[D];
+#pragma unroll
+      for (int j = 0; j < D; ++j) mt[j] = __shfl_sync(0xffffffffu, mu[u][j], top < 0 ? 0 : top);
+      const float lt = odd ? -INFINITY : lmax;
       if (lane == 0) {
         if (odd) {
           lmax = INFINITY;
@@ -325,6 +332,7 @@ __device__ void order_table(const float* __restrict__ centres, const float* __re
         }
         box[kGroupBox * g] = make_float4(lo[0], lo[1], D == 3 ? lo[D - 1] : 0.0f, lmax);
         box[kGroupBox * g + 1] = make_float4(hi[0], hi[1], D == 3 ? hi[D - 1] : 0.0f, 0.0f);
+        box[kGroupBox * g + 2] = make_float4(mt[0], mt[1], D == 3 ? mt[D - 1] : 0.0f, lt);
       }
     }
   }

@@ -255,12 +255,12 @@ __global__ void k_sum_rows(const float* __restrict__ rows, int64_t nrows, int64_
                            float* __restrict__ gbias, const int32_t* __restrict__ perm) {
   int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= width) return;
-  float acc = 0.0f;
-  for (int64_t b = 0; b < nrows; ++b) acc += rows[b * width + m];
+  double acc = 0.0;   // hundreds of rows: FP64 costs nothing beside their loads
+  for (int64_t b = 0; b < nrows; ++b) acc += (double)rows[b * width + m];
   if (m + 1 < width) {
-    if (gw) gw[perm ? perm[m] : m] = acc;
+    if (gw) gw[perm ? perm[m] : m] = (float)acc;
   } else if (gbias) {
-    *gbias = acc;
+    *gbias = (float)acc;
   }
 }
 

@@ -341,7 +341,7 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
   uint32_t* words = reinterpret_cast<uint32_t*>(sm_gw + (GW ? (2 * D + 2) * kTile : 0));
   if (GW)
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
-  float gb = 0.0f;   // warp 0: the bias term of this lane's samples
+  double gb = 0.0;   // warp 0: the bias term of this lane's samples (one number for all of them: FP64)
 
   bool act[K];
   int64_t idx[K];
@@ -385,7 +385,8 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         }
         S[q] = 0ull;
       }
-      near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, false, whole, words, warp, lane);
+      near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearSums, words, warp,
+                         lane);
       __syncthreads();   // the near groups are marked
       near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
                               G);
@@ -438,8 +439,8 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         for (int h = 0; h < NH; ++h) H[q][h] = 0ull;
         S[q] = 0ull;
       }
-      // with the weight gradient, whose sums take phi without its weight, near for those too
-      near_mark<D, W, K>(a.box, a.ngroups, x, act, lo, hi, expanded, gl2e, GW, whole, words, warp, lane);
+      near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearSums, words, warp,
+                         lane);
       __syncthreads();   // the near groups are marked
       NearWalk walk(words, a.ngroups, warp, W);
       int gi = walk.next();
@@ -552,7 +553,7 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
             u2 = fmaf(u[j], u[j], u2);
           }
           if (expanded) f = ex2_approx(-gl2e * u2);
-          gb += cA;
+          gb += (double)cA;
 #pragma unroll
           for (int j = 0; j < D; ++j) {
             GwTerms<D>::put(sm_gw, sidx, j, u[j]);
@@ -566,6 +567,9 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
       }
       __syncthreads();   // every warp has read the reduction buffer before the next pass rebuilds the stages
       if (GW) {          // (and the sample terms are visible)
+        near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearUnweighted,
+                           words, warp, lane);
+        __syncthreads();
         vj_gw_sweep<D, kTile>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, sm_gw, row, lane);
         __syncthreads();   // every warp has walked the groups and read the terms before the next pass marks them
       }
@@ -574,7 +578,7 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
   if (GW && warp == 0) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) gb += __shfl_xor_sync(0xffffffffu, gb, off);
-    if (lane == 0) row[M] = gb;
+    if (lane == 0) row[M] = (float)gb;
   }
   if (warp == 0)
 #pragma unroll
