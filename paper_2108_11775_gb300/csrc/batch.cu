@@ -204,9 +204,9 @@ k_morph_batched(const BatchEnv* __restrict__ envs, const BatchUnit* __restrict__
 }
 
 template <int W, int K>
-static size_t batched_smem(int64_t max_M) {
+static size_t batched_smem() {
   const size_t a = tile_smem_bytes<2, W, K>(), b = tile_smem_bytes<3, W, K>();
-  return (a > b ? a : b) + near_bytes(max_M);
+  return a > b ? a : b;
 }
 
 // ---------------------------------------------------------------- layout
@@ -268,7 +268,7 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   char* base = (char*)ws;
   std::vector<BatchEnv> tab(n);
   std::vector<int64_t> sb(n + 1);
-  int64_t s = 0, cell = 0, max_M = 1;
+  int64_t s = 0, cell = 0;
   for (int e = 0; e < n; ++e) {
     const pdmp_env& E = envs[e];
     BatchEnv& B = tab[e];
@@ -287,7 +287,6 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
     B.T = E.T;
     B.bits = sort_bits(E.field.d, E.N);
     B.cbits = sort_bits(E.field.d, std::min<int64_t>(E.field.M, kOrderChunk));
-    max_M = std::max(max_M, E.field.M);
     B.gamma = E.field.gamma;
     B.bias = E.field.bias;
     B.eta = E.eta;
@@ -324,7 +323,7 @@ cudaError_t batch_prepare(const pdmp_env* envs, int n, int variant, void* ws, pd
   int block = 32 * kVariantW[variant];
 #define PDMP_VARIANT(V, W_, K_)                                                                                      \
   if (variant == V) {                                                                                                \
-    smem = batched_smem<W_, K_>(max_M);                                                                               \
+    smem = batched_smem<W_, K_>();                                                                                    \
     if ((e = cudaFuncSetAttribute(k_morph_batched<W_, K_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) \
       return e;                                                                                                      \
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_morph_batched<W_, K_>, block, smem))) return e; \

@@ -289,128 +289,154 @@ __device__ __forceinline__ bool tile_frame(const float (&x)[K][D], const bool (&
 // A tile with a sample that is not finite has no far groups (its sums must
 // reach it).
 //
-// The near groups are marked in shared memory, one bit each, by all warps of
-// the block together once per sweep; groups past kNearWords * 32 (M > 2^20)
-// count as near.  Every warp then walks the marked groups that are its own.
-// Measured with (1) alone and with both: the morph of 2^20 samples (M = 16,384,
-// T = 50, 2-D) 59.0 and 32.4 ms, the log-density of 2^16 samples 10.3 and 7.4
-// ms, 48 environments 42.2 and 37.3 ms; errors against 64 bits unchanged.
-constexpr int kNearWords = 1024;
-constexpr int kNearExtra = 16;       // words after the marks: the warps' largest ref
+// The near groups of a sweep are listed in shared memory by all warps of the
+// block together, kNearBatch groups (65,536 centres) at a time; every warp then
+// walks the entries that are its own.
+constexpr int kNearBatch = 2048;
 
-__host__ __device__ __forceinline__ int near_words(int ngroups) {
-  const int n = (ngroups + 31) / 32;
-  return n < kNearWords ? n : kNearWords;
-}
-__host__ __device__ __forceinline__ size_t near_bytes(int64_t M) {
-  return ((size_t)(near_words(group_count(M)) + kNearExtra) * 4 + 15) & ~size_t(15);
-}
+struct NearSmem {
+  uint32_t words[kNearBatch / 32];   // a bit per group of the batch
+  float refs[16];                    // the warps' largest ref
+  float state[8];                    // the tile's box and limits, for batches after the first
+  uint16_t list[kNearBatch];         // the near groups, relative to the batch
+};
 
-// what near_mark marks
-enum NearRule { kNearSums, kNearUnweighted, kNearAll };
-
-// Marks the groups that are near the tile's box [lo, hi] (of x, the same in
-// every warp).  kNearSums: rules (1) and (2); kNearUnweighted: rule (1) for sums
-// in which phi stands without its weight; kNearAll: every group.  Block
-// barriers separate it from the walks of the sweep before and of this one.
-template <int D, int W, int K>
-__device__ __forceinline__ void near_mark(const float4* __restrict__ box, int ngroups, int64_t M,
-                                          const float (&x)[K][D], const bool (&act)[K], const float (&lo)[D],
-                                          const float (&hi)[D], bool expanded, float gl2e, NearRule rule,
-                                          uint32_t* words, int warp, int lane) {
-  const int nw = near_words(ngroups);
-  float ref = -INFINITY;
-  if (rule == kNearSums) {
-    // of few groups every warp goes over all (no exchange), of many over its share
-    const bool share = ngroups > 64;
-    for (int g = (share ? warp * 32 : 0) + lane; g < ngroups; g += (share ? W : 1) * 32) {
-      const float4 b = box[kGroupBox * g + 2];
-      const float mu[3] = {b.x, b.y, b.z};
-      float dmin2 = 0.0f, dmax2 = 0.0f;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const float gap = fmaxf(0.0f, fmaxf(mu[j] - hi[j], lo[j] - mu[j]));
-        const float reach = fmaxf(hi[j] - mu[j], mu[j] - lo[j]);
-        dmin2 = fmaf(gap, gap, dmin2);
-        dmax2 = fmaf(reach, reach, dmax2);
-      }
-      ref = fmaxf(ref, fmaf(-gl2e, dmax2, b.w) + 0.5f * lg2_approx(fminf(1.0f, gl2e * dmin2)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, o));
-    if (share) {
-      float* refs = reinterpret_cast<float*>(words + nw);
-      if (lane == 0) refs[warp] = ref;
-      __syncthreads();
-#pragma unroll
-      for (int w = 0; w < W; ++w) ref = fmaxf(ref, refs[w]);
-    }
-  }
-  float R2 = 0.0f;
-  bool odd = false;
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    const float h = 0.5f * (hi[j] - lo[j]);
-    R2 = fmaf(h, h, R2);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-#pragma unroll
-    for (int j = 0; j < D; ++j) odd = odd || (act[k] && !(fabsf(x[k][j]) < INFINITY));
-  odd = __any_sync(0xffffffffu, odd);
-  const float lim1 = odd || rule == kNearAll ? INFINITY : 127.0f + (expanded ? gl2e * R2 : 0.0f);
-  const float lim2 = odd || rule != kNearSums ? INFINITY : 30.0f + lg2_approx((float)M) - ref;
-  for (int q = warp; q < nw; q += W) {
-    const int g = q * 32 + lane;
-    bool near = false;
-    if (g < ngroups) {
-      const float4 b0 = box[kGroupBox * g], b1 = box[kGroupBox * g + 1];
-      const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
-      float d2 = 0.0f;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const float gap = fmaxf(0.0f, fmaxf(blo[j] - hi[j], lo[j] - bhi[j]));
-        d2 = fmaf(gap, gap, d2);
-      }
-      const float y = gl2e * d2, below = y - (rule == kNearUnweighted ? fmaxf(b0.w, 0.0f) : b0.w);
-      // 2 gamma d^2 = 2 ln 2 y
-      const bool far = below > lim1 || (y > 1.0f && below - lg2_approx(fmaf(1.38629436f, y, 1.0f)) > lim2);
-      near = !far;
-    }
-    const uint32_t m = __ballot_sync(0xffffffffu, near);
-    if (lane == 0) words[q] = m;
-  }
-}
-
-// The near groups number own, own + stride, own + 2 stride, ... in order.
+// A warp's share of the list: entries own, own + stride, ...
 struct NearWalk {
-  const uint32_t* words;
-  int ngroups, stride, skip, q;
-  uint32_t m;
-  __device__ __forceinline__ NearWalk(const uint32_t* w, int ng, int own, int st)
-      : words(w), ngroups(ng), stride(st), skip(own), q(-1), m(0) {}
+  const uint16_t* list;
+  int n, i, stride;
+  __device__ __forceinline__ NearWalk(const NearSmem& s, int count, int own, int st)
+      : list(s.list), n(count), i(own), stride(st) {}
   // the next one, or -1 (the same in every lane)
   __device__ __forceinline__ int next() {
-    for (;;) {
-      const int pc = __popc(m);
-      if (pc > skip) {
-        for (; skip > 0; --skip) m &= m - 1;
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        skip = stride - 1;
-        return q * 32 + b;
-      }
-      skip -= pc;
-      if (++q * 32 >= ngroups) {
-        q -= 1;
-        m = 0;
-        return -1;
-      }
-      const int left = ngroups - q * 32;
-      m = q < kNearWords ? words[q] : (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
-    }
+    if (i >= n) return -1;
+    const int g = list[i];
+    i += stride;
+    return g;
   }
 };
+
+// Lists the groups of the range g0 + [0, kNearBatch) below ngroups for which
+// near(g) holds, in order, and returns how many; W warps, two block barriers
+// (the second makes the list visible).
+template <int W, typename F>
+__device__ __forceinline__ int near_list(NearSmem& s, int g0, int ngroups, int warp, int lane, F near) {
+  const int cnt = ngroups - g0 < kNearBatch ? ngroups - g0 : kNearBatch, nw = (cnt + 31) / 32;
+#pragma unroll 2
+  for (int q = warp; q < nw; q += W) {
+    const int g = q * 32 + lane;
+    const uint32_t m = __ballot_sync(0xffffffffu, g < cnt && near(g0 + g));
+    if (lane == 0) s.words[q] = m;
+  }
+  __syncthreads();
+  // exclusive prefix of the words' counts: lane l holds words l and l + 32
+  uint32_t c0 = lane < nw ? __popc(s.words[lane]) : 0u, c1 = lane + 32 < nw ? __popc(s.words[lane + 32]) : 0u;
+  const uint32_t n0 = c0, n1 = c1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t0 = __shfl_up_sync(0xffffffffu, c0, o), t1 = __shfl_up_sync(0xffffffffu, c1, o);
+    if (lane >= o) {
+      c0 += t0;
+      c1 += t1;
+    }
+  }
+  const uint32_t first = __shfl_sync(0xffffffffu, c0, 31), total = first + __shfl_sync(0xffffffffu, c1, 31);
+  c0 -= n0;
+  c1 += first - n1;
+  for (int q = warp; q < nw; q += W) {
+    const uint32_t m = s.words[q], at = __shfl_sync(0xffffffffu, q < 32 ? c0 : c1, q & 31);
+    if (m >> lane & 1u) s.list[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(q * 32 + lane);
+  }
+  __syncthreads();
+  return (int)total;
+}
+
+// what near_tile lists
+enum NearRule { kNearSums, kNearUnweighted, kNearAll };
+
+// Lists the groups of batch g0 that are near the tile's box [lo, hi] (of x, the
+// same in every warp).  kNearSums: rules (1) and (2); kNearUnweighted: rule (1)
+// for sums in which phi stands without its weight; kNearAll: every group.  The
+// first batch (g0 = 0) computes the limits; later ones take them, and the box,
+// from shared memory.  A block barrier must separate it from the walks before.
+template <int D, int W, int K>
+__device__ __forceinline__ int near_tile(const float4* __restrict__ box, int ngroups, int g0, int64_t M,
+                                         const float (&x)[K][D], const bool (&act)[K], float (&lo)[D], float (&hi)[D],
+                                         bool expanded, float gl2e, NearRule rule, NearSmem& s, int warp, int lane) {
+  float lim1, lim2;
+  if (g0 == 0) {
+    float ref = -INFINITY;
+    if (rule == kNearSums) {
+      // of few groups every warp goes over all (no exchange), of many over its share
+      const bool share = ngroups > 64;
+      for (int g = (share ? warp * 32 : 0) + lane; g < ngroups; g += (share ? W : 1) * 32) {
+        const float4 b = box[kGroupBox * g + 2];
+        const float mu[3] = {b.x, b.y, b.z};
+        float dmin2 = 0.0f, dmax2 = 0.0f;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          const float gap = fmaxf(0.0f, fmaxf(mu[j] - hi[j], lo[j] - mu[j]));
+          const float reach = fmaxf(hi[j] - mu[j], mu[j] - lo[j]);
+          dmin2 = fmaf(gap, gap, dmin2);
+          dmax2 = fmaf(reach, reach, dmax2);
+        }
+        ref = fmaxf(ref, fmaf(-gl2e, dmax2, b.w) + 0.5f * lg2_approx(fminf(1.0f, gl2e * dmin2)));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, o));
+      if (share) {
+        if (lane == 0) s.refs[warp] = ref;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) ref = fmaxf(ref, s.refs[w]);
+      }
+    }
+    float R2 = 0.0f;
+    bool odd = false;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      const float h = 0.5f * (hi[j] - lo[j]);
+      R2 = fmaf(h, h, R2);
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int j = 0; j < D; ++j) odd = odd || (act[k] && !(fabsf(x[k][j]) < INFINITY));
+    odd = __any_sync(0xffffffffu, odd);
+    lim1 = odd || rule == kNearAll ? INFINITY : 127.0f + (expanded ? gl2e * R2 : 0.0f);
+    lim2 = odd || rule != kNearSums ? INFINITY : 30.0f + lg2_approx((float)M) - ref;
+    if (ngroups > kNearBatch && threadIdx.x == 0) {
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        s.state[j] = lo[j];
+        s.state[3 + j] = hi[j];
+      }
+      s.state[6] = lim1;
+      s.state[7] = lim2;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      lo[j] = s.state[j];
+      hi[j] = s.state[3 + j];
+    }
+    lim1 = s.state[6];
+    lim2 = s.state[7];
+  }
+  return near_list<W>(s, g0, ngroups, warp, lane, [&](int g) {
+    const float4 b0 = box[kGroupBox * g], b1 = box[kGroupBox * g + 1];
+    const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
+    float d2 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      const float gap = fmaxf(0.0f, fmaxf(blo[j] - hi[j], lo[j] - bhi[j]));
+      d2 = fmaf(gap, gap, d2);
+    }
+    const float y = gl2e * d2, below = y - (rule == kNearUnweighted ? fmaxf(b0.w, 0.0f) : b0.w);
+    // 2 gamma d^2 = 2 ln 2 y
+    return !(below > lim1 || (y > 1.0f && below - lg2_approx(fmaf(1.38629436f, y, 1.0f)) > lim2));
+  });
+}
 
 // Adds the kWarpStage staged records rec to the pair sums S, G of this lane's
 // samples (U: the samples relative to the origin, packed in pairs).
@@ -648,6 +674,24 @@ __device__ __forceinline__ void tile_put_sums(const u64 (&S)[K / 2], const u64 (
   }
 }
 
+// ... or adds them to what is there (its own: a lane adds to what it wrote).
+template <int D, int K>
+__device__ __forceinline__ void tile_add_sums(const u64 (&S)[K / 2], const u64 (&G)[K / 2][D], float4* dst, int lane) {
+#pragma unroll
+  for (int i = 0; i < K / 2; ++i) {
+    float s[2], g0[2], g1[2], g2[2] = {0.0f, 0.0f};
+    upk(S[i], s[0], s[1]);
+    upk(G[i][0], g0[0], g0[1]);
+    upk(G[i][1], g1[0], g1[1]);
+    if (D == 3) upk(G[i][D - 1], g2[0], g2[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4& d = dst[(2 * i + h) * 32 + lane];
+      d = make_float4(d.x + s[h], d.y + g0[h], d.z + g1[h], d.w + g2[h]);
+    }
+  }
+}
+
 __device__ __forceinline__ void add4(float4& acc, const float4& b) {
   acc.x += b.x;
   acc.y += b.y;
@@ -700,23 +744,23 @@ __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t p0, const 
 // The sums S, G over the near groups of one walk, double-buffered through the
 // warp's two stages.  ORIGIN: see fast_tile.
 template <int D, int P, bool ORIGIN>
-__device__ __forceinline__ void near_sweep(const float4* __restrict__ tab, int64_t M, NearWalk walk, bool expanded,
-                                           const float (&o)[D], float gl2e, float4* wraw, u64* wbuf, int lane,
-                                           const u64 (&U)[P][D], u64 (&S)[P], u64 (&G)[P][D]) {
+__device__ __forceinline__ void near_sweep(const float4* __restrict__ tab, int64_t M, int g0, NearWalk walk,
+                                           bool expanded, const float (&o)[D], float gl2e, float4* wraw, u64* wbuf,
+                                           int lane, const u64 (&U)[P][D], u64 (&S)[P], u64 (&G)[P][D]) {
   constexpr int RP = FastRec<D>::kPairs;
   int g = walk.next();
   if (g < 0) return;
   u64* cur = wbuf;
   u64* nxt = wbuf + (size_t)kWarpStage * RP;
-  stage_prefetch<D>(tab, M, (int64_t)g * kWarpStage, wraw, lane);
+  stage_prefetch<D>(tab, M, (int64_t)(g0 + g) * kWarpStage, wraw, lane);
   if (ORIGIN && !expanded)
-    stage_build_origin<D>(M, (int64_t)g * kWarpStage, o, gl2e, wraw, cur, lane);
+    stage_build_origin<D>(M, (int64_t)(g0 + g) * kWarpStage, o, gl2e, wraw, cur, lane);
   else
-    stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, cur, lane);
+    stage_build<D>(M, (int64_t)(g0 + g) * kWarpStage, expanded, o, gl2e, wraw, cur, lane);
   __syncwarp();
   do {
     g = walk.next();
-    const int64_t mn = (int64_t)g * kWarpStage;
+    const int64_t mn = (int64_t)(g0 + g) * kWarpStage;
     if (g >= 0) stage_prefetch<D>(tab, M, mn, wraw, lane);
     if (ORIGIN && !expanded) {
       stage_accumulate_origin<D, P>(cur, U, S, G);
@@ -745,11 +789,11 @@ __host__ __device__ constexpr size_t tile_leaf_bytes() {
   return tile_leaves<W, K>() == W ? 0
                                   : (size_t)tile_leaves<W, K>() / CS * (CS > 1 ? 2 : 1) * (32 * K) * sizeof(float4);
 }
-// + near_bytes(M) at the end
+// (with NearSmem at the end)
 template <int D, int W, int K, int CS = 1>
 __host__ __device__ constexpr size_t tile_smem_bytes() {
   return fast_smem_bytes<D, W, K>() + tile_leaf_bytes<D, W, K, CS>() +
-         (tile_leaves<W, K>() == W ? 0 : (size_t)32 * K * D * sizeof(float));
+         (tile_leaves<W, K>() == W ? 0 : (size_t)32 * K * D * sizeof(float)) + sizeof(NearSmem);
 }
 
 // ORIGIN: tiles too wide for the expanded form take the direct form about the
@@ -772,7 +816,7 @@ __device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t
   float4* wraw = reinterpret_cast<float4*>(smem + fast_region0_bytes<D, W, K>()) + (size_t)warp * kWarpStage * KT;
   float4* leaves = reinterpret_cast<float4*>(smem + fast_smem_bytes<D, W, K>());
   float* xs = reinterpret_cast<float*>(smem + fast_smem_bytes<D, W, K>() + tile_leaf_bytes<D, W, K, CS>());
-  uint32_t* words = reinterpret_cast<uint32_t*>(smem + tile_smem_bytes<D, W, K, CS>());
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(smem + tile_smem_bytes<D, W, K, CS>() - sizeof(NearSmem));
   const float gl2e = a.gamma * kLog2e;
   const bool writer = warp == 0 && crank == 0;
 
@@ -783,7 +827,6 @@ __device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t
   for (int t = 0; t < a.T; ++t) {
     float lo[D], hi[D], o[D];
     const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
-    near_mark<D, W, K>(a.box, a.ngroups, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
     if (ORIGIN && !expanded)
 #pragma unroll
       for (int j = 0; j < D; ++j) {   // the box's centre; 0 when the box is not finite
@@ -812,24 +855,33 @@ __device__ __forceinline__ void fast_tile(const TileArgs& a, int64_t p0, int64_t
         for (int j = 0; j < D; ++j)
           G[i][j] = fma2(pk(x[2 * i][j] - o[j], x[2 * i + 1][j] - o[j]), S[i], mul2(G[i][j], m1));
     };
-    __syncthreads();   // the near groups are marked
     if constexpr (L == W) {
-      near_sweep<D, P, ORIGIN>(a.tab, a.M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U,
-                               S, G);
+      for (int g0 = 0; g0 < a.ngroups; g0 += kNearBatch) {
+        if (g0 > 0) __syncthreads();   // every warp has walked the batch before
+        const int n = near_tile<D, W, K>(a.box, a.ngroups, g0, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, ns, warp,
+                                         lane);
+        near_sweep<D, P, ORIGIN>(a.tab, a.M, g0, NearWalk(ns, n, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S, G);
+      }
       from_origin();
       tile_finish_step<D, W, K, TRACE>(a, t, p0, act, x, o, expanded, S, G, red, warp, lane);
     } else {
       float4* buf = leaves + (CS > 1 ? (t & 1) * (L / CS) * kTile : 0);
-      for (int i = 0; i < L / WT; ++i) {
-        near_sweep<D, P, ORIGIN>(a.tab, a.M, NearWalk(words, a.ngroups, i * WT + crank * W + warp, L), expanded, o,
-                                 gl2e, wraw, wbuf, lane, U, S, G);
-        from_origin();
-        tile_put_sums<D, K>(S, G, buf + (i * W + warp) * kTile, lane);
+      for (int g0 = 0; g0 < a.ngroups; g0 += kNearBatch) {
+        if (g0 > 0) __syncthreads();
+        const int n = near_tile<D, W, K>(a.box, a.ngroups, g0, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, ns, warp,
+                                         lane);
+        for (int i = 0; i < L / WT; ++i) {
+          near_sweep<D, P, ORIGIN>(a.tab, a.M, g0, NearWalk(ns, n, i * WT + crank * W + warp, L), expanded, o, gl2e,
+                                   wraw, wbuf, lane, U, S, G);
+          from_origin();
+          float4* leaf = buf + (i * W + warp) * kTile;
+          if (g0 == 0) tile_put_sums<D, K>(S, G, leaf, lane); else tile_add_sums<D, K>(S, G, leaf, lane);
 #pragma unroll
-        for (int q = 0; q < P; ++q) {
-          S[q] = 0ull;
+          for (int q = 0; q < P; ++q) {
+            S[q] = 0ull;
 #pragma unroll
-          for (int j = 0; j < D; ++j) G[q][j] = 0ull;
+            for (int j = 0; j < D; ++j) G[q][j] = 0ull;
+          }
         }
       }
       // leaf l is slot (l / WT) W + (l % WT) % W of the block of rank (l % WT) / W

@@ -6,6 +6,9 @@
 //
 // Every reduction runs in a fixed order (per-block partials, then one block),
 // so a fit is bit-reproducible.
+//
+// This is the general path (any kind and dimension, from the points as they
+// are); RBF fields in d = 2, 3 run on ordered tiles (fit_rbf.cu).
 #include "field.cuh"
 #include "kernels.cuh"
 
@@ -34,7 +37,7 @@ static int64_t fit_chunks(int64_t n) { return (n + kFitChunk - 1) / kFitChunk; }
 static int64_t fit_nblk(int64_t n) { return (n + kFitThreads - 1) / kFitThreads; }
 static size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-size_t fit_workspace(int64_t M, int64_t n) {
+static size_t general_workspace(int64_t M, int64_t n) {
   size_t b = 0;
   b += align256(sizeof(float) * n) * 2;
   b += align256(sizeof(float) * (M + 1)) * 4;
@@ -42,6 +45,12 @@ size_t fit_workspace(int64_t M, int64_t n) {
   b += align256(sizeof(double) * 8);
   b += align256(sizeof(double) * 2 * fit_nblk(n));
   return b;
+}
+
+// the caller does not say which field it will fit: room for either path
+size_t fit_workspace(int64_t M, int64_t n) {
+  const size_t a = general_workspace(M, n), b = fit_rbf_workspace(M, n);
+  return a > b ? a : b;
 }
 
 static FitWs carve(void* ws, int64_t M, int64_t n) {
@@ -313,6 +322,9 @@ static cudaError_t fit_impl(const FieldArgs& geom, const float* X, const uint8_t
 cudaError_t fit_occupancy(int kind, int d, const FieldArgs& geom, const float* X, const uint8_t* y, int64_t n,
                           float l2, int power_iters, int iters, float* w_out, float* bias_out, float* loss_out,
                           float* alpha_out, void* ws, cudaStream_t st) {
+  // RBF in d = 2, 3: ordered tiles (centres are indexed with 32 bits there)
+  if (kind == PDMP_KIND_RBF && (d == 2 || d == 3) && geom.M <= (int64_t)INT32_MAX)
+    return fit_rbf(d, geom, X, y, n, l2, power_iters, iters, w_out, bias_out, loss_out, alpha_out, ws, st);
 #define PDMP_CASE(KD, DD)                                                                                    \
   if (kind == KD && d == DD)                                                                                 \
     return fit_impl<KD, DD>(geom, X, y, n, l2, power_iters, iters, w_out, bias_out, loss_out, alpha_out, ws, \

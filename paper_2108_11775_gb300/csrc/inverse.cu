@@ -149,7 +149,7 @@ __device__ __forceinline__ void inverse_tile(const TileArgs& a, float tol, int m
   float* zs = reinterpret_cast<float*>(smem + fast_smem_bytes<D, W, K>());   // kTile x D
   float* ds = zs + kTile * D;    // the corrections of the two steps undone before (warm start),
   float* ds2 = ds + kTile * D;   // kTile x D each
-  uint32_t* words = reinterpret_cast<uint32_t*>(ds2 + kTile * D);
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(ds2 + kTile * D);
   float y[K][D];
   bool act[K];
   tile_load<D, K>(a, p0, p_end, lane, y, act);
@@ -189,10 +189,12 @@ __device__ __forceinline__ void inverse_tile(const TileArgs& a, float tol, int m
         }
         S[i] = 0ull;
       }
-      near_mark<D, W, K>(a.box, a.ngroups, a.M, y, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
-      __syncthreads();   // the near groups are marked
-      near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
-                              G);
+      for (int g0 = 0; g0 < a.ngroups; g0 += kNearBatch) {
+        if (g0 > 0) __syncthreads();   // every warp has walked the batch before
+        const int n = near_tile<D, W, K>(a.box, a.ngroups, g0, M, y, act, lo, hi, expanded, gl2e, kNearSums, ns, warp,
+                                         lane);
+        near_sweep<D, P, false>(a.tab, M, g0, NearWalk(ns, n, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S, G);
+      }
       __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
 #pragma unroll
       for (int i = 0; i < P; ++i) {
@@ -295,8 +297,8 @@ k_morph_inverse_fast(TileArgs a, float tol, int maxit, int32_t* __restrict__ ite
 template <int D, int K>
 static cudaError_t launch_inverse_shape(const TileArgs& a, float tol, int maxit, int32_t* iters,
                                         unsigned long long* work, cudaStream_t st) {
-  const size_t smem =
-      fast_smem_bytes<D, 4, K>() + 3 * (size_t)Shape<4, K>::kTile * D * sizeof(float) + near_bytes(a.M);
+  constexpr size_t smem =
+      fast_smem_bytes<D, 4, K>() + 3 * (size_t)Shape<4, K>::kTile * D * sizeof(float) + sizeof(NearSmem);
   cudaError_t e =
       cudaFuncSetAttribute(k_morph_inverse_fast<D, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -155,6 +155,11 @@ cudaError_t residual_threshold(int d, const FieldArgs& fa, const float* x0, int6
                                float* tau_r, float* xT, void* ws, cudaStream_t st);
 
 size_t fit_workspace(int64_t M, int64_t n);
+// RBF, d = 2, 3 on ordered points and centres (fit_rbf.cu); M < 2^31
+size_t fit_rbf_workspace(int64_t M, int64_t n);
+cudaError_t fit_rbf(int d, const FieldArgs& geom, const float* X, const uint8_t* y, int64_t n, float l2,
+                    int power_iters, int iters, float* w_out, float* bias_out, float* loss_out, float* alpha_out,
+                    void* ws, cudaStream_t st);
 cudaError_t fit_occupancy(int kind, int d, const FieldArgs& geom, const float* X, const uint8_t* y, int64_t n,
                           float l2, int power_iters, int iters, float* w_out, float* bias_out, float* loss_out,
                           float* alpha_out, void* ws, cudaStream_t st);

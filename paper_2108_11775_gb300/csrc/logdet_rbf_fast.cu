@@ -173,15 +173,14 @@ __device__ __forceinline__ void ld_stage_accumulate(const u64* rec, bool expande
   }
 }
 
-// One sweep over the near groups of centres for the tile's samples x (words:
-// near_bytes; every warp over its own groups, double-buffered stages); the per-warp sums S, G, H land in red
+// One sweep over the near groups of centres for the tile's samples x (every warp over its own groups, double-buffered stages); the per-warp sums S, G, H land in red
 // ([W][NS][kTile] floats, aliasing the stages).  Returns whether the tile took
 // the expanded form, with its origin in o.  Ends with a block barrier after
 // the sums are written; the caller must pass another barrier before the next
 // sweep rebuilds the stages.
 template <int D, int K = kLdK<D>>
 __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][D], const bool (&act)[K],
-                                         float (&o)[D], unsigned char* smem, uint32_t* words, int warp, int lane) {
+                                         float (&o)[D], unsigned char* smem, NearSmem& ns, int warp, int lane) {
   using L = LdRbf<D, K>;
   constexpr int W = L::kW, P = K / 2, RP = L::kPairs, NH = L::kH;
   constexpr int NS = L::kSums, kTile = L::kTile, KT = FastRec<D>::kTab;
@@ -192,7 +191,6 @@ __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][
   const float gl2e = a.gamma * kLog2e;
   float lo[D], hi[D];
   const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
-  near_mark<D, W, K>(a.box, a.ngroups, a.M, x, act, lo, hi, expanded, gl2e, kNearSums, words, warp, lane);
   u64 U[P][D], S[P], G[P][D], H[P][NH];
 #pragma unroll
   for (int i = 0; i < P; ++i) {
@@ -205,22 +203,25 @@ __device__ __forceinline__ bool ld_sweep(const TileArgs& a, const float (&x)[K][
     for (int h = 0; h < NH; ++h) H[i][h] = 0ull;
     S[i] = 0ull;
   }
-  __syncthreads();   // the near groups are marked
-  NearWalk walk(words, a.ngroups, warp, W);
-  int g = walk.next();
-  if (g >= 0) {
-    stage_prefetch<D>(a.tab, M, (int64_t)g * kWarpStage, wraw, lane);
-    ld_stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
-  }
-  __syncwarp();
-  for (int st = 0; g >= 0; st ^= 1) {
-    g = walk.next();
-    if (g >= 0) stage_prefetch<D>(a.tab, M, (int64_t)g * kWarpStage, wraw, lane);
-    ld_stage_accumulate<D, P>(wbuf + (size_t)st * kWarpStage * RP, expanded, gl2e, U, S, G, H);
-    if (g >= 0)
-      ld_stage_build<D>(M, (int64_t)g * kWarpStage, expanded, o, gl2e, wraw, wbuf + (size_t)(st ^ 1) * kWarpStage * RP,
-                        lane);
+  for (int g0 = 0; g0 < a.ngroups; g0 += kNearBatch) {
+    if (g0 > 0) __syncthreads();   // every warp has walked the batch before
+    const int n = near_tile<D, W, K>(a.box, a.ngroups, g0, M, x, act, lo, hi, expanded, gl2e, kNearSums, ns, warp, lane);
+    NearWalk walk(ns, n, warp, W);
+    int g = walk.next();
+    if (g >= 0) {
+      stage_prefetch<D>(a.tab, M, (int64_t)(g0 + g) * kWarpStage, wraw, lane);
+      ld_stage_build<D>(M, (int64_t)(g0 + g) * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
+    }
     __syncwarp();
+    for (int st = 0; g >= 0; st ^= 1) {
+      g = walk.next();
+      const int64_t mn = (int64_t)(g0 + g) * kWarpStage;
+      if (g >= 0) stage_prefetch<D>(a.tab, M, mn, wraw, lane);
+      ld_stage_accumulate<D, P>(wbuf + (size_t)st * kWarpStage * RP, expanded, gl2e, U, S, G, H);
+      if (g >= 0)
+        ld_stage_build<D>(M, mn, expanded, o, gl2e, wraw, wbuf + (size_t)(st ^ 1) * kWarpStage * RP, lane);
+      __syncwarp();
+    }
   }
   __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
 #pragma unroll
@@ -324,7 +325,7 @@ k_logdet_rbf_fast(TileArgs a, float* __restrict__ logdet) {
   const float* red = reinterpret_cast<const float*>(smem);
   const int64_t p0 = (int64_t)blockIdx.x * kTile;
   const float eta = a.eta;
-  uint32_t* words = reinterpret_cast<uint32_t*>(smem + ld_rbf_smem<D>());
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(smem + ld_rbf_smem<D>());
 
   float x[K][D];
   bool act[K];
@@ -339,7 +340,7 @@ k_logdet_rbf_fast(TileArgs a, float* __restrict__ logdet) {
 
   for (int t = 0; t < a.T; ++t) {
     float o[D];
-    const bool expanded = ld_sweep<D>(a, x, act, o, smem, words, warp, lane);
+    const bool expanded = ld_sweep<D>(a, x, act, o, smem, ns, warp, lane);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       float shat, gs[D], hs[D][D];
@@ -395,7 +396,7 @@ k_log_density_rbf_fast(TileArgs a, float tol, int maxit, float* __restrict__ log
   float* zs = reinterpret_cast<float*>(smem + ld_rbf_smem<D, K>());   // kTile x D: the step's target z
   float* ds = zs + kTile * D;    // the corrections of the two steps undone before, kTile x D each
   float* ds2 = ds + kTile * D;
-  uint32_t* words = reinterpret_cast<uint32_t*>(ds2 + kTile * D);
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(ds2 + kTile * D);
 
   float y[K][D];
   bool act[K];
@@ -433,7 +434,7 @@ k_log_density_rbf_fast(TileArgs a, float tol, int maxit, float* __restrict__ log
     bool moving = true;
     while (moving && it < maxit) {
       float o[D];
-      const bool expanded = ld_sweep<D, K>(a, y, act, o, smem, words, warp, lane);
+      const bool expanded = ld_sweep<D, K>(a, y, act, o, smem, ns, warp, lane);
       bool mv = false;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
@@ -515,7 +516,7 @@ static cudaError_t launch_logdet_rbf_fast(const FieldArgs& fa, const float* x0, 
   a.perm_base = 0;
   a.N = N;
   a.xT = xT;
-  const size_t smem = ld_rbf_smem<D>() + near_bytes(fa.M);
+  constexpr size_t smem = ld_rbf_smem<D>() + sizeof(NearSmem);
   e = cudaFuncSetAttribute(k_logdet_rbf_fast<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((N + LdRbf<D>::kTile - 1) / LdRbf<D>::kTile);
@@ -526,8 +527,8 @@ static cudaError_t launch_logdet_rbf_fast(const FieldArgs& fa, const float* x0, 
 template <int D, int K>
 static cudaError_t launch_log_density_shape(const TileArgs& a, float tol, int maxit, float* ld, int32_t* iters,
                                             unsigned long long* work, cudaStream_t st) {
-  const size_t smem =
-      ld_rbf_smem<D, K>() + 3 * (size_t)LdRbf<D, K>::kTile * D * sizeof(float) + near_bytes(a.M);
+  constexpr size_t smem =
+      ld_rbf_smem<D, K>() + 3 * (size_t)LdRbf<D, K>::kTile * D * sizeof(float) + sizeof(NearSmem);
   cudaError_t e =
       cudaFuncSetAttribute(k_log_density_rbf_fast<D, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -57,7 +57,7 @@ size_t morph_rbf_fast_workspace(int d, int64_t M, int64_t N) { return rbf_order_
 
 template <int D, bool TRACE, int K, int CS>
 static cudaError_t launch_shape(const TileArgs& a, int64_t N, cudaStream_t st) {
-  const size_t smem = tile_smem_bytes<D, 4, K, CS>() + near_bytes(a.M);
+  constexpr size_t smem = tile_smem_bytes<D, 4, K, CS>();
   const unsigned blocks = (unsigned)((N + Shape<4, K>::kTile - 1) / Shape<4, K>::kTile) * CS;
   auto fn = k_morph_rbf_fast<D, TRACE, K, CS>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

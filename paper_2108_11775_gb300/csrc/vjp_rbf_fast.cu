@@ -79,7 +79,7 @@ struct GwTerms {
 // the tile's sample terms), a feature a lane and kGwFeatures groups at a time;
 // adds each feature's sum to row (in table order).
 template <int D, int kTile>
-__device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int64_t M, NearWalk walk,
+__device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int64_t M, int g0, NearWalk walk,
                                             bool expanded, const float* o, float gl2e, const float* sm,
                                             float* __restrict__ row, int lane) {
   constexpr int TP = GwTerms<D>::kPairs;
@@ -90,7 +90,7 @@ __device__ __forceinline__ void vj_gw_sweep(const float4* __restrict__ tab, int6
 #pragma unroll
     for (int f = 0; f < F; ++f) {
       const int g = walk.next();
-      mf[f] = g < 0 ? M : (int64_t)g * kGroup + lane;
+      mf[f] = g < 0 ? M : (int64_t)(g0 + g) * kGroup + lane;
     }
     if (mf[0] >= M && __all_sync(0xffffffffu, mf[0] >= M)) break;
     u64 cst[F], bm[F][D], A[F], Q[F][D];
@@ -338,7 +338,7 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
   // the forward's S, G (cross-warp totals) at the segment's states: [kseg][1 + D][kTile]
   float* sgc = seg + (size_t)kseg * kTile * D;
   float* sm_gw = sgc + (use_cache ? (size_t)kseg * (1 + D) * kTile : 0);   // [kTile / 2][2D + 2] packed pairs
-  uint32_t* words = reinterpret_cast<uint32_t*>(sm_gw + (GW ? (2 * D + 2) * kTile : 0));
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(sm_gw + (GW ? (2 * D + 2) * kTile : 0));
   if (GW)
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
   double gb = 0.0;   // warp 0: the bias term of this lane's samples (one number for all of them: FP64)
@@ -385,11 +385,12 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         }
         S[q] = 0ull;
       }
-      near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearSums, words, warp,
-                         lane);
-      __syncthreads();   // the near groups are marked
-      near_sweep<D, P, false>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S,
-                              G);
+      for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
+        if (gb0 > 0) __syncthreads();   // every warp has walked the batch before
+        const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                         whole ? kNearAll : kNearSums, ns, warp, lane);
+        near_sweep<D, P, false>(a.tab, M, gb0, NearWalk(ns, n, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S, G);
+      }
       tile_finish_step<D, W, K, false>(a, 0, p0, act, x, o, expanded, S, G, reinterpret_cast<float4*>(red), warp,
                                        lane);
       if (use_cache && i >= pre) {
@@ -439,28 +440,30 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         for (int h = 0; h < NH; ++h) H[q][h] = 0ull;
         S[q] = 0ull;
       }
-      near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearSums, words, warp,
-                         lane);
-      __syncthreads();   // the near groups are marked
-      NearWalk walk(words, a.ngroups, warp, W);
-      int gi = walk.next();
-      if (gi >= 0) {
-        stage_prefetch<D>(a.tab, M, (int64_t)gi * kWarpStage, wraw, lane);
-        vj_stage_build<D>(M, (int64_t)gi * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
-      }
-      __syncwarp();
-      for (int st = 0; gi >= 0; st ^= 1) {
-        gi = walk.next();
-        const u64* cur = wbuf + (size_t)st * kWarpStage * RP;
-        if (gi >= 0) stage_prefetch<D>(a.tab, M, (int64_t)gi * kWarpStage, wraw, lane);
-        if (have)
-          vj_stage_accumulate<D, P, false>(cur, expanded, gl2e, U, V, S, G, H);
-        else
-          vj_stage_accumulate<D, P, true>(cur, expanded, gl2e, U, V, S, G, H);
-        if (gi >= 0)
-          vj_stage_build<D>(M, (int64_t)gi * kWarpStage, expanded, o, gl2e, wraw,
-                            wbuf + (size_t)(st ^ 1) * kWarpStage * RP, lane);
+      for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
+        if (gb0 > 0) __syncthreads();
+        const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                         whole ? kNearAll : kNearSums, ns, warp, lane);
+        NearWalk walk(ns, n, warp, W);
+        int gi = walk.next();
+        if (gi >= 0) {
+          stage_prefetch<D>(a.tab, M, (int64_t)(gb0 + gi) * kWarpStage, wraw, lane);
+          vj_stage_build<D>(M, (int64_t)(gb0 + gi) * kWarpStage, expanded, o, gl2e, wraw, wbuf, lane);
+        }
         __syncwarp();
+        for (int st = 0; gi >= 0; st ^= 1) {
+          gi = walk.next();
+          const int64_t mn = (int64_t)(gb0 + gi) * kWarpStage;
+          const u64* cur = wbuf + (size_t)st * kWarpStage * RP;
+          if (gi >= 0) stage_prefetch<D>(a.tab, M, mn, wraw, lane);
+          if (have)
+            vj_stage_accumulate<D, P, false>(cur, expanded, gl2e, U, V, S, G, H);
+          else
+            vj_stage_accumulate<D, P, true>(cur, expanded, gl2e, U, V, S, G, H);
+          if (gi >= 0)
+            vj_stage_build<D>(M, mn, expanded, o, gl2e, wraw, wbuf + (size_t)(st ^ 1) * kWarpStage * RP, lane);
+          __syncwarp();
+        }
       }
       __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
       float* rw = red + (size_t)warp * NS * kTile;
@@ -566,13 +569,13 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         for (int j = 0; j < D; ++j) g[k][j] = g[k][j] - eta * fmaf(d1, hv[j], d2 * gd * gs[j]);
       }
       __syncthreads();   // every warp has read the reduction buffer before the next pass rebuilds the stages
-      if (GW) {          // (and the sample terms are visible)
-        near_mark<D, W, K>(a.box, a.ngroups, M, x, act, lo, hi, expanded, gl2e, whole ? kNearAll : kNearUnweighted,
-                           words, warp, lane);
-        __syncthreads();
-        vj_gw_sweep<D, kTile>(a.tab, M, NearWalk(words, a.ngroups, warp, W), expanded, o, gl2e, sm_gw, row, lane);
-        __syncthreads();   // every warp has walked the groups and read the terms before the next pass marks them
-      }
+      if (GW)            // (and the sample terms are visible)
+        for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
+          const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                           whole ? kNearAll : kNearUnweighted, ns, warp, lane);
+          vj_gw_sweep<D, kTile>(a.tab, M, gb0, NearWalk(ns, n, warp, W), expanded, o, gl2e, sm_gw, row, lane);
+          __syncthreads();   // every warp has walked the groups and read the terms
+        }
     }
   }
   if (GW && warp == 0) {
@@ -613,7 +616,7 @@ static cudaError_t launch_vjp_rbf_fast(const FieldArgs& fa, const float* x0, int
   const void* fn = want ? reinterpret_cast<const void*>(k_vjp_rbf_fast<D, true>)
                         : reinterpret_cast<const void*>(k_vjp_rbf_fast<D, false>);
   // cache the recompute's S and G when the extra shared memory keeps as many blocks on an SM
-  const size_t nb = near_bytes(fa.M);
+  const size_t nb = sizeof(NearSmem);
   const size_t smem0 = vj_rbf_smem<D>(k, want, false) + nb, smem1 = vj_rbf_smem<D>(k, want, true) + nb;
   int b0 = 0, b1 = 0;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
