@@ -38,7 +38,7 @@ D, M, N, T = 2, 16384, 1 << 20, 50
 # ncu captures that must stay small (well under a second of replay per pass)
 SMALL = {"N": 1 << 18, "T": 3}
 L2_FLUSH_BYTES = 256 << 20
-LAUNCHES_PER_MORPH = 9
+LAUNCHES_PER_MORPH = 7
 FP32_LANES_PER_SM = 128           # FP32 pipe width per SM per clock
 MUFU_EX2_PER_SM = 32              # measured ex2 throughput per SM per clock on GB300
 MUFU_SINCOS_PER_SM = 15.6         # measured sin (or cos) throughput per SM per clock on GB300
@@ -293,7 +293,7 @@ def run_ours(args, world, rank, local):
                                    f"128 FP32 lanes / (2d+2) FP32 operations per feature",
                      "kernel_pipe_peak": pipe_peak, "kernel_pipe_frac": achieved / pipe_peak},
         "clocks": clk.summary(),
-        # per step: the ordered centre table, 7 kernels of the samples' sort, the morph kernel
+        # per step: the ordered centre table, 5 kernels of the samples' sort, the morph kernel
         "gpu_launches": args.steps * LAUNCHES_PER_MORPH,
         "wall_s_timed": wall1 - wall0,
     }
@@ -365,7 +365,7 @@ def extra_batched(pdmp, torch, n_sms, pk):
     return {"value": work / t, "unit": "feature-evals/s", "ms_per_launch": 1e3 * t, "work": work,
             "roofline_frac": (work / t) / (work / t_peak), "variant": best,
             "variant_ms": [round(v, 3) for v in times], "launch": "CUDA graph of one pdmp_morph_batched",
-            "gpu_launches_per_run": 11}
+            "gpu_launches_per_run": 8}
 
 
 def extra_cspace(pdmp, torch, fld, info, n=1 << 16, t_steps=20, links=7, per_link=4):
@@ -387,7 +387,7 @@ def extra_cspace(pdmp, torch, fld, info, n=1 << 16, t_steps=20, links=7, per_lin
     b = links * per_link
     return {"value": n * t_steps / t, "unit": "sample-steps/s", "ms": 1e3 * t, "N": n, "T": t_steps,
             "joints": links, "body_points": b, "feature_evals_per_s": n * t_steps * b * M / t, "eta": eta, "L_q": Lq,
-            "launches_per_step": 11}
+            "launches_per_step": 9}
 
 
 def extra_sampler(pdmp, torch, fld, eta, batch=1 << 16, capacity=1 << 20, t_steps=50):
@@ -466,7 +466,7 @@ def extra_inverse(pdmp, torch, fld, x0, xT, eta, n_sms, pk, n=1 << 18, n_direct=
             "mean_iterations_per_step": evals / (n * T * M), "round_trip_max_abs": rt,
             "direct_kernel": {"value": float(wd.item()) / td, "N": n_direct, "ms": 1e3 * td},
             "log_density": {"samples_per_s": n / tl, "ms": 1e3 * tl},
-            "launches_per_call": 9}
+            "launches_per_call": 7}
 
 
 def extra_tanh_net(pdmp, torch, n_sms, pk, d=2, H=64, n=1 << 20, t_steps=50):

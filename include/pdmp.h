@@ -578,6 +578,14 @@ pdmp_status pdmp_logdet(const pdmp_field* f, const float* x0, int64_t N, int32_t
 pdmp_status pdmp_occupancy_query(const pdmp_field* f, const float* x, int64_t N, float* c, float* s, float* grad,
                                  void* stream);
 
+/* The same with a device workspace of pdmp_occupancy_query_workspace(f, N)
+ * bytes (16-byte aligned; 0: this request gains nothing from one), with which
+ * long sweeps of RBF fields in d = 2, 3 run on spatially sorted tiles.
+ * ws = NULL is pdmp_occupancy_query. */
+size_t pdmp_occupancy_query_workspace(const pdmp_field* f, int64_t N);
+pdmp_status pdmp_occupancy_query_ws(const pdmp_field* f, const float* x, int64_t N, float* c, float* s, float* grad,
+                                    void* ws, size_t ws_bytes, void* stream);
+
 /* label[n] = 1 iff x[n] lies in some closed axis-aligned box:
  * lo_j <= x_j <= hi_j on every axis, compared exactly in float32.
  * boxes: nb x 2d (lo_0..lo_{d-1}, hi_0..hi_{d-1}); nb >= 0; 1 <= d <= 8. */

@@ -120,6 +120,7 @@ def lib():
                 "pdmp_morph_inverse": [_FP, _P, _i64, _i32, _f32, _f32, _i32, _P, _P, _P, _sz, _P, _P],
                 "pdmp_log_density": [_FP, _P, _i64, _i32, _f32, _P, _P, _f32, _i32, _P, _P, _P, _sz, _P],
                 "pdmp_occupancy_query": [_FP, _P, _i64, _P, _P, _P, _P],
+                "pdmp_occupancy_query_ws": [_FP, _P, _i64, _P, _P, _P, _P, _sz, _P],
                 "pdmp_box_labels": [_i32, _P, _i64, _P, _i64, _P, _P],
                 "pdmp_lipschitz_bound": [_FP, ctypes.POINTER(_f64), ctypes.POINTER(_f64), _i32,
                                          ctypes.POINTER(_f64), ctypes.POINTER(_f64), _P],
@@ -136,6 +137,8 @@ def lib():
             L.pdmp_cspace_workspace.restype = _sz
             L.pdmp_morph_culled_workspace.argtypes = [_FP, _i64]
             L.pdmp_morph_culled_workspace.restype = _sz
+            L.pdmp_occupancy_query_workspace.argtypes = [_FP, _i64]
+            L.pdmp_occupancy_query_workspace.restype = _sz
             L.pdmp_morph_vjp_workspace.argtypes = [_FP, _i64, _i32, _i32, _i32]
             L.pdmp_morph_vjp_workspace.restype = _sz
             L.pdmp_fit_workspace.argtypes = [_i64, _i64]
@@ -640,8 +643,11 @@ def occupancy_query(field: DeviceField, x: torch.Tensor, want=("c", "s", "grad")
     s = torch.empty(N, device=x.device, dtype=torch.float32) if "s" in want else None
     g = torch.empty(N, d, device=x.device, dtype=torch.float32) if "grad" in want else None
     f = field.struct()
-    st = lib().pdmp_occupancy_query(ctypes.byref(f), _ptr(x, shape=(N, d), name="x"), N, _ptr(c), _ptr(s), _ptr(g),
-                                    _stream())
+    # long sweeps of 2-D / 3-D RBF fields run on sorted tiles, which want a workspace
+    nbytes = int(lib().pdmp_occupancy_query_workspace(ctypes.byref(f), N))
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=x.device) if nbytes else None
+    st = lib().pdmp_occupancy_query_ws(ctypes.byref(f), _ptr(x, shape=(N, d), name="x"), N, _ptr(c), _ptr(s), _ptr(g),
+                                       ctypes.c_void_p(ws.data_ptr()) if nbytes else None, nbytes, _stream())
     _check(st, "pdmp_occupancy_query")
     return {"c": c, "s": s, "grad": g}
 

@@ -117,6 +117,10 @@ cudaError_t log_density_rbf_fast(int d, const FieldArgs& fa, const float* z, int
                                  int maxit, float* y, float* ld, int32_t* iters, unsigned long long* work, void* ws,
                                  cudaStream_t st);
 
+// c, s, grad c (any may be NULL) at N points on sorted tiles (RBF, d = 2, 3)
+size_t query_rbf_fast_workspace(int d, int64_t M, int64_t N);
+cudaError_t query_rbf_fast(int d, const FieldArgs& fa, const float* x, int64_t N, float* c, float* s, float* grad,
+                           void* ws, cudaStream_t st);
 cudaError_t occupancy_query(int kind, int d, const FieldArgs& fa, const float* x, int64_t N, float* c, float* s,
                             float* grad, cudaStream_t st);
 cudaError_t box_labels(int d, const float* boxes, int64_t nb, const float* x, int64_t N, uint8_t* label,

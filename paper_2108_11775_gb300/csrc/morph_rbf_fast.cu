@@ -136,6 +136,27 @@ cudaError_t morph_rbf_fast(int d, const FieldArgs& fa, const float* x0, int64_t 
   return cudaErrorInvalidValue;
 }
 
+__global__ void k_query_c(const float* __restrict__ s, int64_t N, float* __restrict__ c) {
+  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n < N) c[n] = sigmoid_f(s[n]);
+}
+
+// s needs N floats of its own when the caller wants c alone
+size_t query_rbf_fast_workspace(int d, int64_t M, int64_t N) {
+  return morph_rbf_fast_workspace(d, M, N) + ((sizeof(float) * (size_t)N + 255) & ~size_t(255));
+}
+
+cudaError_t query_rbf_fast(int d, const FieldArgs& fa, const float* x, int64_t N, float* c, float* s, float* grad,
+                           void* ws, cudaStream_t st) {
+  if (c != nullptr && s == nullptr) s = (float*)((char*)ws + morph_rbf_fast_workspace(d, fa.M, N));
+  // one step with the update discarded, as grad_rbf_fast
+  cudaError_t e = d == 2 ? launch_fast<2>(fa, x, N, 1, 0.0f, nullptr, nullptr, 0, nullptr, nullptr, ws, st, s, grad)
+                         : launch_fast<3>(fa, x, N, 1, 0.0f, nullptr, nullptr, 0, nullptr, nullptr, ws, st, s, grad);
+  if (e != cudaSuccess || c == nullptr) return e;
+  k_query_c<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(s, N, c);
+  return cudaGetLastError();
+}
+
 cudaError_t grad_rbf_fast(int d, const FieldArgs& fa, const float* x, int64_t N, float* g, void* ws,
                           cudaStream_t st) {
   // one step with the update discarded: the per-sample gradient output only

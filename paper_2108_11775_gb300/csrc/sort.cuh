@@ -88,11 +88,13 @@ __device__ __forceinline__ uint32_t cell_coord(float v, float lo, float hi, floa
   return cell_at(v, lo, cell_scale(lo, hi, cells), cells);
 }
 
+constexpr int kSortBoxes = 304;   // blocks of a sort's first launch at most
+
 struct SortWs {
   int bits;           // grid cells per axis = 2^bits
   int64_t cells;      // 2^(d * bits)
   int64_t nchunks;    // scan chunks
-  uint32_t* box;      // 2d ordered-float bounds
+  float* boxes;       // kSortBoxes partial bounding boxes
   uint32_t* keys;     // N cell keys
   int32_t* perm;      // N: sorted position -> original index
   uint32_t* counts;   // cells
