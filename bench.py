@@ -365,7 +365,7 @@ def extra_batched(pdmp, torch, n_sms, pk):
     return {"value": work / t, "unit": "feature-evals/s", "ms_per_launch": 1e3 * t, "work": work,
             "roofline_frac": (work / t) / (work / t_peak), "variant": best,
             "variant_ms": [round(v, 3) for v in times], "launch": "CUDA graph of one pdmp_morph_batched",
-            "gpu_launches_per_run": 8}
+            "gpu_launches_per_run": 10}
 
 
 def extra_cspace(pdmp, torch, fld, info, n=1 << 16, t_steps=20, links=7, per_link=4):

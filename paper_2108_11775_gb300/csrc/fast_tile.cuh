@@ -356,13 +356,15 @@ enum NearRule { kNearSums, kNearUnweighted, kNearAll };
 
 // Lists the groups of batch g0 that are near the tile's box [lo, hi] (of x, the
 // same in every warp).  kNearSums: rules (1) and (2); kNearUnweighted: rule (1)
-// for sums in which phi stands without its weight; kNearAll: every group.  The
+// for sums in which phi stands without its weight; kNearAll: every group.  CS >
+// 1: only every CS-th group, those of block crank of a cluster.  The
 // first batch (g0 = 0) computes the limits; later ones take them, and the box,
 // from shared memory.  A block barrier must separate it from the walks before.
-template <int D, int W, int K>
+template <int D, int W, int K, int CS = 1>
 __device__ __forceinline__ int near_tile(const float4* __restrict__ box, int ngroups, int g0, int64_t M,
                                          const float (&x)[K][D], const bool (&act)[K], float (&lo)[D], float (&hi)[D],
-                                         bool expanded, float gl2e, NearRule rule, NearSmem& s, int warp, int lane) {
+                                         bool expanded, float gl2e, NearRule rule, NearSmem& s, int warp, int lane,
+                                         int crank = 0) {
   float lim1, lim2;
   if (g0 == 0) {
     float ref = -INFINITY;
@@ -424,6 +426,7 @@ __device__ __forceinline__ int near_tile(const float4* __restrict__ box, int ngr
     lim2 = s.state[7];
   }
   return near_list<W>(s, g0, ngroups, warp, lane, [&](int g) {
+    if (CS > 1 && (g & (CS - 1)) != crank) return false;
     const float4 b0 = box[kGroupBox * g], b1 = box[kGroupBox * g + 1];
     const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
     float d2 = 0.0f;

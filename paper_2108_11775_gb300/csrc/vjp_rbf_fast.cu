@@ -314,66 +314,118 @@ __device__ __forceinline__ void vj_stage_accumulate(const u64* rec, bool expande
   }
 }
 
-template <int D, bool GW>
+// A tile's state x and cotangent g live in shared memory (xs, gs); every warp
+// loads all of the tile's samples for a sweep, and each thread finishes its own
+// one or two samples after it (samples threadIdx.x and + 128).
+//
+// CS > 1: a cluster of CS blocks shares the tile, each taking every CS-th group
+// of centres; the blocks add up their sums through each other's shared memory
+// and all finish every sample alike, so only the sums travel.
+template <int D, bool GW, int CS>
 __global__ void __launch_bounds__(VjRbf<D>::kW * 32, 3)
 k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT,
                float* __restrict__ g0, float* __restrict__ rows, int use_cache) {
   constexpr int W = VjRbf<D>::kW, K = VjRbf<D>::kK, P = K / 2, RP = VjRbf<D>::kPairs;
-  constexpr int NS = VjRbf<D>::kSums, kTile = VjRbf<D>::kTile, KT = FastRec<D>::kTab;
+  constexpr int NS = VjRbf<D>::kSums, kTile = VjRbf<D>::kTile, KT = FastRec<D>::kTab, NH = VjRbf<D>::kH;
+  constexpr int kOwn = (kTile + 32 * W - 1) / (32 * W);   // samples a thread finishes
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = (int)(blockIdx.x / CS), crank = (int)(blockIdx.x % CS);
   u64* wbuf = reinterpret_cast<u64*>(smem) + (size_t)warp * 2 * kWarpStage * RP;
   float* red = reinterpret_cast<float*>(smem);   // [W][NS][kTile], aliases the stages after a pass's last stage
+  float4* red4 = reinterpret_cast<float4*>(smem);          // the recompute's: [W][kTile]
   float4* wraw = reinterpret_cast<float4*>(smem + vj_rbf_region0<D>()) + (size_t)warp * kWarpStage * KT;
   float* seg = reinterpret_cast<float*>(smem + vj_rbf_region0<D>() +
-                                        (size_t)W * kWarpStage * KT * sizeof(float4));   // [kseg][kTile][D]
-  const int64_t p0 = (int64_t)blockIdx.x * kTile;
+                                        (size_t)W * kWarpStage * KT * sizeof(float4));   // [kseg][D][kTile]
+  const int64_t p0 = (int64_t)tile * kTile;
   const int64_t N = a.N, M = a.M;
   const float gamma = a.gamma, gl2e = gamma * kLog2e, eta = a.eta;
   // with the weight gradient a ragged tile visits every group: its empty slots sit at 0, where the expanded
   // sums can overflow, and what they then add to the row has to stay what it is without far groups
   const bool whole = GW && p0 + kTile > N;
-  // weight gradient: this block's row of rows[blocks][M + 1] (features in table order) and the sample terms after the segment
-  float* row = GW ? rows + (int64_t)blockIdx.x * (M + 1) : nullptr;
+  // weight gradient: this tile's row of rows[tiles][M + 1] (features in table order) and the sample terms after
+  // the segment
+  float* row = GW ? rows + (int64_t)tile * (M + 1) : nullptr;
   // the forward's S, G (cross-warp totals) at the segment's states: [kseg][1 + D][kTile]
   float* sgc = seg + (size_t)kseg * kTile * D;
   float* sm_gw = sgc + (use_cache ? (size_t)kseg * (1 + D) * kTile : 0);   // [kTile / 2][2D + 2] packed pairs
-  NearSmem& ns = *reinterpret_cast<NearSmem*>(sm_gw + (GW ? (2 * D + 2) * kTile : 0));
-  if (GW)
-    for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
-  double gb = 0.0;   // warp 0: the bias term of this lane's samples (one number for all of them: FP64)
+  float* xs = sm_gw + (GW ? (2 * D + 2) * kTile : 0);      // [D][kTile]
+  float* gs = xs + D * kTile;                              // [D][kTile]
+  float* ex = gs + D * kTile;                              // [NS][kTile], CS > 1: this block's sums
+  NearSmem& ns = *reinterpret_cast<NearSmem*>(ex + (CS > 1 ? NS * kTile : 0));
+  if (GW)   // this block's features
+    for (int64_t g = crank; g * kGroup < M; g += CS)
+      if (threadIdx.x < kGroup && g * kGroup + threadIdx.x < M) row[g * kGroup + threadIdx.x] = 0.0f;
+  double gb = 0.0;   // the bias term of this thread's samples (one number for all of them: FP64)
 
   bool act[K];
-  int64_t idx[K];
-  float g[K][D], x[K][D];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int64_t p = p0 + k * 32 + lane;
-    act[k] = p < N;
-    idx[k] = act[k] ? (int64_t)a.perm[p] - a.perm_base : 0;
+  for (int k = 0; k < K; ++k) act[k] = p0 + k * 32 + lane < N;
+  int64_t idx[kOwn];   // this thread's samples
+  bool mine[kOwn];
 #pragma unroll
-    for (int j = 0; j < D; ++j) g[k][j] = act[k] ? gT[idx[k] * D + j] : 0.0f;
+  for (int h = 0; h < kOwn; ++h) {
+    const int sm = threadIdx.x + h * 32 * W;
+    mine[h] = sm < kTile && p0 + sm < N;
+    idx[h] = mine[h] ? (int64_t)a.perm[p0 + sm] - a.perm_base : 0;
+    if (sm < kTile)
+#pragma unroll
+      for (int j = 0; j < D; ++j) gs[j * kTile + sm] = mine[h] ? gT[idx[h] * D + j] : 0.0f;
   }
+
+  // CS > 1: total of sum q (v: this block's) of sample sm over the cluster, in the blocks' order
+  bool pending = false;   // the others may still read this block's sums
+  auto publish = [&]() {
+    if (CS > 1 && pending) cluster_wait();
+  };
+  auto exchange = [&]() {
+    if (CS > 1) cluster_barrier();
+  };
+  auto release = [&]() {
+    if (CS > 1) {
+      cluster_arrive();
+      pending = true;
+    }
+  };
+  auto total = [&](int q, int sm) {
+    float v = 0.0f;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) {
+      const float t = __uint_as_float(cluster_load(cluster_addr(&ex[q * kTile + sm], r)));
+      v = r == 0 ? t : v + t;
+    }
+    return v;
+  };
 
   const int nseg = a.T / kseg;
   for (int sgi = nseg - 1; sgi >= 0; --sgi) {
     const float* src = (sgi == 0 || ckpt == nullptr) ? a.x0 : ckpt + (int64_t)(sgi - 1) * N * D;
 #pragma unroll
-    for (int k = 0; k < K; ++k)
+    for (int h = 0; h < kOwn; ++h) {
+      const int sm = threadIdx.x + h * 32 * W;
+      if (sm < kTile)
 #pragma unroll
-      for (int j = 0; j < D; ++j) x[k][j] = act[k] ? src[idx[k] * D + j] : 0.0f;
+        for (int j = 0; j < D; ++j) xs[j * kTile + sm] = mine[h] ? src[idx[h] * D + j] : 0.0f;
+    }
     const int pre = (sgi > 0 && ckpt == nullptr) ? sgi * kseg : 0;   // no checkpoints: recompute from x0
     for (int i = 0; i < pre + kseg; ++i) {
       if (i >= pre) {
-        if (warp == 0)
 #pragma unroll
-          for (int k = 0; k < K; ++k)
+        for (int h = 0; h < kOwn; ++h) {
+          const int sm = threadIdx.x + h * 32 * W;
+          if (sm < kTile)
 #pragma unroll
-            for (int j = 0; j < D; ++j) seg[((i - pre) * kTile + k * 32 + lane) * D + j] = x[k][j];
+            for (int j = 0; j < D; ++j) seg[((i - pre) * D + j) * kTile + sm] = xs[j * kTile + sm];
+        }
         if (i == pre + kseg - 1) break;
       }
+      __syncthreads();   // the states are visible, the reduction buffer is read
       // one forward step of the tile (every warp holds all its samples)
-      float lo[D], hi[D], o[D];
+      float x[K][D], lo[D], hi[D], o[D];
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[k][j] = xs[j * kTile + k * 32 + lane];
       const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
       u64 U[P][D], S[P], G[P][D];
 #pragma unroll
@@ -387,46 +439,65 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
       }
       for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
         if (gb0 > 0) __syncthreads();   // every warp has walked the batch before
-        const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
-                                         whole ? kNearAll : kNearSums, ns, warp, lane);
+        const int n = near_tile<D, W, K, CS>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                             whole ? kNearAll : kNearSums, ns, warp, lane, crank);
         near_sweep<D, P, false>(a.tab, M, gb0, NearWalk(ns, n, warp, W), expanded, o, gl2e, wraw, wbuf, lane, U, S, G);
       }
-      tile_finish_step<D, W, K, false>(a, 0, p0, act, x, o, expanded, S, G, reinterpret_cast<float4*>(red), warp,
-                                       lane);
-      if (use_cache && i >= pre) {
-        // the step's totals, added in the finish's order, for the Hessian-vector pass at the same state
-        const float4* r4 = reinterpret_cast<const float4*>(red);
-        if (warp == 0)
+      __syncthreads();   // every warp has finished its centres before the reduction buffer overwrites the stages
+      tile_put_sums<D, K>(S, G, red4 + warp * kTile, lane);
+      __syncthreads();
+      float4 acc[kOwn];
+      publish();
 #pragma unroll
-          for (int k = 0; k < K; ++k) {
-            float4 acc = r4[k * 32 + lane];
+      for (int h = 0; h < kOwn; ++h) {
+        const int sm = threadIdx.x + h * 32 * W;
+        acc[h] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (sm >= kTile) continue;
+        acc[h] = red4[sm];
 #pragma unroll
-            for (int w = 1; w < W; ++w) {
-              const float4 b = r4[w * kTile + k * 32 + lane];
-              acc.x += b.x;
-              acc.y += b.y;
-              acc.z += b.z;
-              acc.w += b.w;
-            }
-            float* dst = sgc + (size_t)(i - pre) * (1 + D) * kTile + k * 32 + lane;
-            dst[0] = acc.x;
-            dst[kTile] = acc.y;
-            dst[2 * kTile] = acc.z;
-            if (D == 3) dst[3 * kTile] = acc.w;
-          }
-        __syncthreads();   // read before the next step's stages overwrite the buffer
+        for (int w = 1; w < W; ++w) add4(acc[h], red4[w * kTile + sm]);
+        if (CS > 1) {
+          ex[sm] = acc[h].x;
+          ex[kTile + sm] = acc[h].y;
+          ex[2 * kTile + sm] = acc[h].z;
+          if (D == 3) ex[3 * kTile + sm] = acc[h].w;
+        }
       }
+      exchange();
+#pragma unroll
+      for (int h = 0; h < kOwn; ++h) {
+        const int sm = threadIdx.x + h * 32 * W;
+        if (sm >= kTile) continue;
+        if (CS > 1) acc[h] = make_float4(total(0, sm), total(1, sm), total(2, sm), D == 3 ? total(3, sm) : 0.0f);
+        if (use_cache && i >= pre) {   // for the Hessian-vector pass at the same state
+          float* dst = sgc + (size_t)(i - pre) * (1 + D) * kTile + sm;
+          dst[0] = acc[h].x;
+          dst[kTile] = acc[h].y;
+          dst[2 * kTile] = acc[h].z;
+          if (D == 3) dst[3 * kTile] = acc[h].w;
+        }
+        float xo[1][D];
+        const bool ao[1] = {mine[h]};
+#pragma unroll
+        for (int j = 0; j < D; ++j) xo[0][j] = xs[j * kTile + sm];
+        tile_update<D, 1, false>(a, 0, p0, ao, xo, o, expanded, acc[h], 0, false, lane);
+#pragma unroll
+        for (int j = 0; j < D; ++j) xs[j * kTile + sm] = xo[0][j];
+      }
+      release();
     }
-    __syncthreads();   // the segment's states (and totals) are visible to every warp
     for (int i = kseg - 1; i >= 0; --i) {
+      __syncthreads();   // the segment's states, the cotangents (and the weight gradient's marks and terms) are done
+      float x[K][D], g[K][D], lo[D], hi[D], o[D];
 #pragma unroll
       for (int k = 0; k < K; ++k)
 #pragma unroll
-        for (int j = 0; j < D; ++j) x[k][j] = seg[(i * kTile + k * 32 + lane) * D + j];
-      float lo[D], hi[D], o[D];
+        for (int j = 0; j < D; ++j) {
+          x[k][j] = seg[(i * D + j) * kTile + k * 32 + lane];
+          g[k][j] = gs[j * kTile + k * 32 + lane];
+        }
       const bool expanded = tile_frame<D, K>(x, act, gl2e, lo, hi, o);
       const bool have = use_cache && i < kseg - 1;   // S and G at this state from the recompute
-      constexpr int NH = VjRbf<D>::kH;
       u64 U[P][D], V[P][D], S[P], G[P][D], H[P][NH];
 #pragma unroll
       for (int q = 0; q < P; ++q) {
@@ -442,8 +513,8 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
       }
       for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
         if (gb0 > 0) __syncthreads();
-        const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
-                                         whole ? kNearAll : kNearSums, ns, warp, lane);
+        const int n = near_tile<D, W, K, CS>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                             whole ? kNearAll : kNearSums, ns, warp, lane, crank);
         NearWalk walk(ns, n, warp, W);
         int gi = walk.next();
         if (gi >= 0) {
@@ -489,106 +560,166 @@ k_vjp_rbf_fast(TileArgs a, int kseg, const float* __restrict__ ckpt, const float
         }
       }
       __syncthreads();
+      float sums[kOwn][NS];
+      publish();
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        float sum[NS];
+      for (int h = 0; h < kOwn; ++h) {
+        const int sm = threadIdx.x + h * 32 * W;
+        if (sm >= kTile) continue;
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
           if (have && q <= D) {   // the recompute's totals at this state
-            sum[q] = sgc[((size_t)i * (1 + D) + q) * kTile + k * 32 + lane];
+            sums[h][q] = sgc[((size_t)i * (1 + D) + q) * kTile + sm];
             continue;
           }
-          float v = red[q * kTile + k * 32 + lane];
+          float v = red[q * kTile + sm];
 #pragma unroll
-          for (int w = 1; w < W; ++w) v += red[((size_t)w * NS + q) * kTile + k * 32 + lane];
-          sum[q] = v;
+          for (int w = 1; w < W; ++w) v += red[((size_t)w * NS + q) * kTile + sm];
+          sums[h][q] = v;
+          if (CS > 1) ex[q * kTile + sm] = v;
+        }
+      }
+      exchange();
+#pragma unroll
+      for (int h = 0; h < kOwn; ++h) {
+        const int sm = threadIdx.x + h * 32 * W;
+        if (sm >= kTile) continue;
+        if (CS > 1)
+#pragma unroll
+          for (int q = 0; q < NS; ++q)
+            if (!(have && q <= D)) sums[h][q] = total(q, sm);
+        const float(&sum)[NS] = sums[h];
+        float xo[D], go[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          xo[j] = seg[(i * D + j) * kTile + sm];
+          go[j] = gs[j * kTile + sm];
         }
         const float Ss = sum[0];
-        float shat, gs[D], hv[D];
+        float shat, gsv[D], hv[D];
         if (expanded) {
           float u[D], u2 = 0.0f, uv = 0.0f;
 #pragma unroll
           for (int j = 0; j < D; ++j) {
-            u[j] = x[k][j] - o[j];
+            u[j] = xo[j] - o[j];
             u2 = fmaf(u[j], u[j], u2);
-            uv = fmaf(u[j], g[k][j], uv);
+            uv = fmaf(u[j], go[j], uv);
           }
           const float f = ex2_approx(-gl2e * u2);
           shat = f * Ss;
           float vG = 0.0f;   // K = sum e' (c . v) = v . G
 #pragma unroll
-          for (int j = 0; j < D; ++j) vG = fmaf(g[k][j], sum[1 + j], vG);
+          for (int j = 0; j < D; ++j) vG = fmaf(go[j], sum[1 + j], vG);
 #pragma unroll
           for (int j = 0; j < D; ++j) {
             float Hv = 0.0f;   // Kc_j = (H v)_j, H from its lower triangle
 #pragma unroll
             for (int i2 = 0; i2 < D; ++i2) {
               const int q = j >= i2 ? j * (j + 1) / 2 + i2 : i2 * (i2 + 1) / 2 + j;
-              Hv = fmaf(sum[1 + D + q], g[k][i2], Hv);
+              Hv = fmaf(sum[1 + D + q], go[i2], Hv);
             }
             const float usg = fmaf(u[j], Ss, -sum[1 + j]);                  // u S - G
-            gs[j] = -2.0f * gamma * (f * usg);
+            gsv[j] = -2.0f * gamma * (f * usg);
             const float m = fmaf(uv, usg, -fmaf(u[j], vG, -Hv));            // (u.v)(uS-G) - (u K - Kc)
-            hv[j] = 4.0f * gamma * gamma * f * m - 2.0f * gamma * f * Ss * g[k][j];
+            hv[j] = 4.0f * gamma * gamma * f * m - 2.0f * gamma * f * Ss * go[j];
           }
         } else {
           shat = Ss;
 #pragma unroll
           for (int j = 0; j < D; ++j) {
-            gs[j] = -2.0f * gamma * sum[1 + j];
-            hv[j] = 4.0f * gamma * gamma * sum[1 + D + j] - 2.0f * gamma * Ss * g[k][j];
+            gsv[j] = -2.0f * gamma * sum[1 + j];
+            hv[j] = 4.0f * gamma * gamma * sum[1 + D + j] - 2.0f * gamma * Ss * go[j];
           }
         }
         float d1, d2;
         sigmoid_d12(shat + a.bias, d1, d2);
         float gd = 0.0f;
 #pragma unroll
-        for (int j = 0; j < D; ++j) gd = fmaf(gs[j], g[k][j], gd);
-        if (GW && warp == 0) {   // the sample's weight-gradient terms, with g_{t+1}
-          const int sidx = k * 32 + lane;
-          const float cA = act[k] ? -eta * d2 * gd : 0.0f, cB = act[k] ? -eta * d1 : 0.0f;
+        for (int j = 0; j < D; ++j) gd = fmaf(gsv[j], go[j], gd);
+        if (GW) {   // the sample's weight-gradient terms, with g_{t+1}
+          const float cA = mine[h] ? -eta * d2 * gd : 0.0f, cB = mine[h] ? -eta * d1 : 0.0f;
           float u[D], ug = 0.0f, f = 1.0f, u2 = 0.0f;
 #pragma unroll
           for (int j = 0; j < D; ++j) {
             // direct form: o = 0; an empty slot sits at the origin, where phi / f <= 1 stays finite
-            u[j] = act[k] ? x[k][j] - o[j] : 0.0f;
-            ug = fmaf(u[j], g[k][j], ug);
+            u[j] = mine[h] ? xo[j] - o[j] : 0.0f;
+            ug = fmaf(u[j], go[j], ug);
             u2 = fmaf(u[j], u[j], u2);
           }
           if (expanded) f = ex2_approx(-gl2e * u2);
           gb += (double)cA;
 #pragma unroll
           for (int j = 0; j < D; ++j) {
-            GwTerms<D>::put(sm_gw, sidx, j, u[j]);
-            GwTerms<D>::put(sm_gw, sidx, D + 1 + j, f * (2.0f * gamma * cB * g[k][j]));
+            GwTerms<D>::put(sm_gw, sm, j, u[j]);
+            GwTerms<D>::put(sm_gw, sm, D + 1 + j, f * (2.0f * gamma * cB * go[j]));
           }
-          GwTerms<D>::put(sm_gw, sidx, D, f * fmaf(-2.0f * gamma * cB, ug, cA));
-          GwTerms<D>::put(sm_gw, sidx, 2 * D + 1, 0.0f);
+          GwTerms<D>::put(sm_gw, sm, D, f * fmaf(-2.0f * gamma * cB, ug, cA));
+          GwTerms<D>::put(sm_gw, sm, 2 * D + 1, 0.0f);
         }
 #pragma unroll
-        for (int j = 0; j < D; ++j) g[k][j] = g[k][j] - eta * fmaf(d1, hv[j], d2 * gd * gs[j]);
+        for (int j = 0; j < D; ++j) gs[j * kTile + sm] = go[j] - eta * fmaf(d1, hv[j], d2 * gd * gsv[j]);
       }
-      __syncthreads();   // every warp has read the reduction buffer before the next pass rebuilds the stages
-      if (GW)            // (and the sample terms are visible)
+      release();
+      if (GW) {
+        __syncthreads();   // the sample terms are visible
         for (int gb0 = 0; gb0 < a.ngroups; gb0 += kNearBatch) {
-          const int n = near_tile<D, W, K>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
-                                           whole ? kNearAll : kNearUnweighted, ns, warp, lane);
+          if (gb0 > 0) __syncthreads();
+          const int n = near_tile<D, W, K, CS>(a.box, a.ngroups, gb0, M, x, act, lo, hi, expanded, gl2e,
+                                               whole ? kNearAll : kNearUnweighted, ns, warp, lane, crank);
           vj_gw_sweep<D, kTile>(a.tab, M, gb0, NearWalk(ns, n, warp, W), expanded, o, gl2e, sm_gw, row, lane);
-          __syncthreads();   // every warp has walked the groups and read the terms
         }
+      }
     }
+    __syncthreads();   // the cotangents and the last terms are read before the next segment
   }
-  if (GW && warp == 0) {
+  publish();           // no block leaves while another may read its sums
+  if (GW && crank == 0) {
+    double* sh = reinterpret_cast<double*>(smem);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) gb += __shfl_xor_sync(0xffffffffu, gb, off);
-    if (lane == 0) row[M] = (float)gb;
+    if (lane == 0) sh[warp] = gb;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < W; ++w) gb += sh[w];
+      row[M] = (float)gb;
+    }
   }
-  if (warp == 0)
+  if (crank == 0)
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (act[k])
+    for (int h = 0; h < kOwn; ++h)
+      if (mine[h])
 #pragma unroll
-        for (int j = 0; j < D; ++j) g0[idx[k] * D + j] = g[k][j];
+        for (int j = 0; j < D; ++j) g0[idx[h] * D + j] = gs[j * kTile + threadIdx.x + h * 32 * W];
+}
+
+template <int D, bool GW, int CS>
+static cudaError_t launch_vjp_shape(const TileArgs& a, int64_t tiles, int k, const float* ckpt, const float* gT,
+                                    float* g0, float* rows, cudaStream_t st) {
+  auto fn = k_vjp_rbf_fast<D, GW, CS>;
+  // cache the recompute's S and G when the extra shared memory keeps as many blocks on an SM
+  const size_t more = (2 * D + (CS > 1 ? VjRbf<D>::kSums : 0)) * VjRbf<D>::kTile * sizeof(float) + sizeof(NearSmem);
+  const size_t smem0 = vj_rbf_smem<D>(k, GW, false) + more, smem1 = vj_rbf_smem<D>(k, GW, true) + more;
+  int b0 = 0, b1 = 0;
+  const bool fits = smem1 <= 227 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(fits ? smem1 : smem0));
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, fn, VjRbf<D>::kW * 32, smem0);
+  if (e == cudaSuccess && fits) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, fn, VjRbf<D>::kW * 32, smem1);
+  if (e != cudaSuccess) return e;
+  const int use_cache = b1 >= b0 && b1 > 0 ? 1 : 0;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)(tiles * CS));
+  c.blockDim = dim3(VjRbf<D>::kW * 32);
+  c.dynamicSmemBytes = use_cache ? smem1 : smem0;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = CS > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&c, fn, a, k, ckpt, gT, g0, rows, use_cache);
 }
 
 template <int D>
@@ -612,29 +743,23 @@ static cudaError_t launch_vjp_rbf_fast(const FieldArgs& fa, const float* x0, int
   a.perm_base = 0;
   a.N = N;
   a.kck = 1;
-  const bool want = rows != nullptr;
-  const void* fn = want ? reinterpret_cast<const void*>(k_vjp_rbf_fast<D, true>)
-                        : reinterpret_cast<const void*>(k_vjp_rbf_fast<D, false>);
-  // cache the recompute's S and G when the extra shared memory keeps as many blocks on an SM
-  const size_t nb = sizeof(NearSmem);
-  const size_t smem0 = vj_rbf_smem<D>(k, want, false) + nb, smem1 = vj_rbf_smem<D>(k, want, true) + nb;
-  int b0 = 0, b1 = 0;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, fn, VjRbf<D>::kW * 32, smem0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, fn, VjRbf<D>::kW * 32, smem1);
-  if (e != cudaSuccess) return e;
-  const int use_cache = b1 >= b0 && b1 > 0 ? 1 : 0;
-  const size_t smem = use_cache ? smem1 : smem0;
-  const unsigned blocks = (unsigned)vjp_rbf_fast_blocks(D, N);
-  if (!want) {
-    k_vjp_rbf_fast<D, false><<<blocks, VjRbf<D>::kW * 32, smem, st>>>(a, k, ckpt, gT, g0, nullptr, use_cache);
-    return cudaGetLastError();
+  const int64_t tiles = vjp_rbf_fast_blocks(D, N);
+  // Blocks per tile, measured with d/dw (M = 8192, T = 50, k = 5; forward and VJP in ms for 1, 2, 4, 8 blocks):
+  // 59 tiles 21.1, 11.4, 8.1, 7.9; 117 12.6, 9.7, 7.8, 8.8; 235 22.0, 16.6, 14.4, 15.4; 782 tiles (M = 1000) 1.7,
+  // 2.0, 3.0, 5.2.
+  const int cs = tiles <= 114 ? 8 : (tiles <= 304 ? 4 : (tiles <= 456 ? 2 : 1));
+  if (rows == nullptr) {
+    if (cs == 8) return launch_vjp_shape<D, false, 8>(a, tiles, k, ckpt, gT, g0, nullptr, st);
+    if (cs == 4) return launch_vjp_shape<D, false, 4>(a, tiles, k, ckpt, gT, g0, nullptr, st);
+    if (cs == 2) return launch_vjp_shape<D, false, 2>(a, tiles, k, ckpt, gT, g0, nullptr, st);
+    return launch_vjp_shape<D, false, 1>(a, tiles, k, ckpt, gT, g0, nullptr, st);
   }
-  k_vjp_rbf_fast<D, true><<<blocks, VjRbf<D>::kW * 32, smem, st>>>(a, k, ckpt, gT, g0, rows, use_cache);
-  e = cudaGetLastError();
+  if (cs == 8) e = launch_vjp_shape<D, true, 8>(a, tiles, k, ckpt, gT, g0, rows, st);
+  else if (cs == 4) e = launch_vjp_shape<D, true, 4>(a, tiles, k, ckpt, gT, g0, rows, st);
+  else if (cs == 2) e = launch_vjp_shape<D, true, 2>(a, tiles, k, ckpt, gT, g0, rows, st);
+  else e = launch_vjp_shape<D, true, 1>(a, tiles, k, ckpt, gT, g0, rows, st);
   if (e != cudaSuccess) return e;
-  return sum_vjp_rows(rows, (int64_t)blocks, fa.M + 1, gw, gbias, st, ord.cperm);
+  return sum_vjp_rows(rows, tiles, fa.M + 1, gw, gbias, st, ord.cperm);
 }
 
 int64_t vjp_rbf_fast_blocks(int d, int64_t N) {

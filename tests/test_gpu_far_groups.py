@@ -57,14 +57,15 @@ def test_morph_and_vjp_with_far_groups(d, M, N):
     assert max_abs(ld[idx], oracle.logdet(f, x0[idx], T, eta)[0]) <= 1e-4 * T
 
 
-@pytest.mark.parametrize("d", [2, 3])
-def test_weight_gradient_in_the_callers_order(d):
+@pytest.mark.parametrize("d,tiles", [(2, 3), (3, 3), (2, 115), (3, 305), (2, 457)])
+def test_weight_gradient_in_the_callers_order(d, tiles):
     """Rows are summed in the centres' own order and handed back in the caller's;
-    features of zero weight have a gradient too.  N is a multiple of the tile."""
+    features of zero weight have a gradient too.  Whole tiles, as many as take
+    clusters of 8, 4 and 2 blocks and single ones."""
     f = wide_field(d, 1500, 20.0 if d == 2 else 8.0)
     lo, hi = np.zeros(d), np.full(d, 20.0 if d == 2 else 8.0)
     eta, _ = rbf_eta(f, lo, hi, cells=24 if d == 2 else 8)
-    N, T, k = 768, 4, 2
+    N, T, k = tiles * (256 if d == 2 else 192), 4, 2
     x0 = wl.uniform_box(d, 3, N, lo, hi)
     gT = wl.f32(wl.rng(d, wl.S_COTANGENT).standard_normal((N, d)))
     _, gw, gb = pdmp.morph_vjp(pdmp.DeviceField.from_host(f), dev(x0), T, eta, k, dev(gT), want_param_grad=True)
