@@ -22,7 +22,8 @@
 // A block of 4 warps owns 4 x 32 samples; each warp sweeps all features
 // for its own 32 (two 16-row tiles), the features staged for the whole
 // block in double-buffered shared-memory stages of 128 (one bulk copy each).  A
-// sample's state stays in the warp's shared memory for all T steps.
+// sample's state stays in the warp's shared memory for all T steps.  Morphs of
+// few tiles spread a tile over a cluster (RmShare).
 #include "fast_tile.cuh"
 #include "kernels.cuh"
 
@@ -232,12 +233,40 @@ __device__ __forceinline__ void rm_split(u64 a, u64& hi, u64& lo) {
   lo = fma2(hi, mone, a);
 }
 
+// A morph of few samples spreads a tile over a cluster of CS blocks: every
+// block holds the tile's samples, sweeps its own range of the table's stages,
+// and adds up the blocks' sums through each other's shared memory, in the
+// blocks' order, so that all of them take the same step.
+struct RmShare {
+  int crank, st0, st1;
+  float* ex;       // per warp [32 rows][8]: the sums of grad s in columns 0 .. 6, of s in 7
+  bool pending;    // the others may still read this block's sums
+};
+
+__device__ __forceinline__ RmShare rm_share(int cs, int nstage, float* ex) {
+  if (cs == 1) return RmShare{0, 0, nstage, ex, false};
+  const int r = (int)(blockIdx.x % cs);
+  return RmShare{r, nstage * r / cs, nstage * (r + 1) / cs, ex, false};
+}
+
+__device__ __forceinline__ float2 cluster_load2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
+template <int CS>
+__device__ __forceinline__ void rm_leave(RmShare& sh) {   // no block leaves while another may read its sums
+  if (CS > 1 && sh.pending) cluster_wait();
+}
+
 // One pass over all features for the warp's 32 samples.  In:
 // A fragments of [x, 1] (ah, al) and, with HVP, of [v, 0] (vh, vl).  Out:
 // S (packed partial logits: row g / g + 8, features 2t / 2t + 1), G (D
 // fragments of grad s) and, with HVP, P (D fragments of
 // sum_m cos(theta_m) (omega_m . v / 2 pi) (-w_m omega_m) = (Hess s) v / 2 pi).
-// Block-wide: every warp of the block makes the same sequence of passes.
+// Block-wide: every warp of the block makes the same sequence of passes.  tab
+// and nstage: the stages of this block (all of them without a cluster).
 template <bool HVP>
 __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nstage, float* sm,
                                          const uint32_t (&ah)[kRmRows][4], const uint32_t (&al)[kRmRows][4],
@@ -338,9 +367,47 @@ __device__ __forceinline__ float rm_logit(const u64 (&S)[kRmRows][2], int r, int
   return s;
 }
 
+// The totals over the cluster's blocks: s (without the bias) of rows r * 16 + g +
+// 8 hh, and G.
+template <int CS>
+__device__ __forceinline__ void rm_combine(RmShare& sh, const u64 (&S)[kRmRows][2], float (&s)[kRmRows][2],
+                                           float (&G)[kRmRows][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int r = 0; r < kRmRows; ++r)
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) s[r][hh] = rm_logit(S, r, hh);
+  float* ex = sh.ex + (threadIdx.x >> 5) * (kRmWarpSamples * 8);
+  if (sh.pending) cluster_wait();
+#pragma unroll
+  for (int r = 0; r < kRmRows; ++r)
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh)
+      *reinterpret_cast<float2*>(ex + (r * 16 + g + 8 * hh) * 8 + 2 * t) =
+          make_float2(G[r][2 * hh], t == 3 ? s[r][hh] : G[r][2 * hh + 1]);
+  cluster_barrier();
+#pragma unroll
+  for (int r = 0; r < kRmRows; ++r)
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const float* e = ex + (r * 16 + g + 8 * hh) * 8 + 2 * t;
+      float2 a = make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int q = 0; q < CS; ++q) {
+        const float2 v = cluster_load2(cluster_addr(e, q));
+        a = q == 0 ? v : make_float2(a.x + v.x, a.y + v.y);
+      }
+      s[r][hh] = __shfl_sync(0xffffffffu, a.y, lane | 3);
+      G[r][2 * hh] = a.x;
+      G[r][2 * hh + 1] = t == 3 ? 0.0f : a.y;   // column 7 is no dimension
+    }
+  cluster_arrive();
+  sh.pending = true;
+}
+
 // One Euler step of the warp's 32 samples held in xs ([32][8], column 7 = 1).
-template <int D, bool TRACE>
-__device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, int nstage, float* sm, float* xs,
+template <int D, bool TRACE, int CS = 1>
+__device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, RmShare& sh, float* sm, float* xs,
                                               float bias, float eta, int64_t s0, int64_t N, int step,
                                               float* __restrict__ traj, float* __restrict__ steps) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -348,14 +415,16 @@ __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, int
   rm_frags(xs, g, t, ah, al);
   float G[kRmRows][4], P[kRmRows][4];
   u64 S[kRmRows][2];
-  rm_sweep<false>(tab, nstage, sm, ah, al, ah, al, S, G, P);
+  rm_sweep<false>(CS == 1 ? tab : tab + (size_t)sh.st0 * kRmStageFloats, CS == 1 ? sh.st1 : sh.st1 - sh.st0, sm, ah,
+                  al, ah, al, S, G, P);
+  float s[kRmRows][2];
+  if (CS > 1) rm_combine<CS>(sh, S, s, G);
 #pragma unroll
   for (int r = 0; r < kRmRows; ++r) {
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
-      const float s = rm_logit(S, r, hh);
       float d1, d2;
-      sigmoid_d12(s + bias, d1, d2);
+      sigmoid_d12((CS == 1 ? rm_logit(S, r, hh) : s[r][hh]) + bias, d1, d2);
       const float c = -eta * d1;
       const int row = r * 16 + g + 8 * hh;
       const int64_t n = s0 + row;
@@ -364,7 +433,7 @@ __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, int
         const int j = 2 * t + e;
         if (j < D) {
           const float inc = __fmul_rn(c, G[r][2 * hh + e]);
-          if (TRACE && n < N) {
+          if (TRACE && sh.crank == 0 && n < N) {
             traj[((int64_t)step * N + n) * D + j] = xs[row * 8 + j];
             steps[((int64_t)step * N + n) * D + j] = inc;
           }
@@ -398,7 +467,7 @@ __device__ __forceinline__ void rm_store_rows(const float* xs, int64_t s0, int64
   }
 }
 
-template <int D, bool TRACE>
+template <int D, bool TRACE, int CS>
 __global__ void __launch_bounds__(kRmWarps * 32, 4)
 k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
                 float eta, float* __restrict__ xT, float* __restrict__ ckpt, int kck, float* __restrict__ traj,
@@ -408,13 +477,16 @@ k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const flo
   rm_stage_init();
   const int warp = threadIdx.x >> 5;
   float* xs = sm + 2 * kRmStageFloats + warp * (kRmWarpSamples * 8);   // [32 samples][8]: x, 0 .., 1
-  const int64_t s0 = (int64_t)blockIdx.x * kRmSamples + warp * kRmWarpSamples;
+  RmShare sh = rm_share(CS, nstage, sm + 2 * kRmStageFloats + kRmWarps * (kRmWarpSamples * 8));
+  const int64_t s0 = (int64_t)(blockIdx.x / CS) * kRmSamples + warp * kRmWarpSamples;
   rm_load_rows<D>(x0, s0, N, 1.0f, xs);
   for (int step = 0; step < T; ++step) {
-    rm_euler_step<D, TRACE>(tab, nstage, sm, xs, bias, eta, s0, N, step, traj, steps);
-    if (ckpt != nullptr && (step + 1) % kck == 0)
+    rm_euler_step<D, TRACE, CS>(tab, sh, sm, xs, bias, eta, s0, N, step, traj, steps);
+    if (ckpt != nullptr && (step + 1) % kck == 0 && sh.crank == 0)
       rm_store_rows<D>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
   }
+  rm_leave<CS>(sh);
+  if (sh.crank > 0) return;
   if (xT) rm_store_rows<D>(xs, s0, N, xT);
   if (TRACE) rm_store_rows<D>(xs, s0, N, traj + (int64_t)T * N * D);
 }
@@ -513,6 +585,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
   float gb_acc = 0.0f;
   const int64_t s0 = (int64_t)blockIdx.x * kRmSamples + warp * kRmWarpSamples;
+  RmShare one = rm_share(1, nstage, nullptr);
   rm_load_rows<D>(gT, s0, N, 0.0f, gs);
   const float twopi = k2PiHi;
   const int nseg = T / kseg;
@@ -520,7 +593,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
     if (sgi == 0 || ckpt == nullptr) {
       rm_load_rows<D>(x0, s0, N, 1.0f, seg);
       for (int q = 0; q < sgi * kseg; ++q)
-        rm_euler_step<D, false>(tab, nstage, sm, seg, bias, eta, s0, N, 0, nullptr, nullptr);
+        rm_euler_step<D, false>(tab, one, sm, seg, bias, eta, s0, N, 0, nullptr, nullptr);
     } else {
       rm_load_rows<D>(ckpt + (int64_t)(sgi - 1) * N * D, s0, N, 1.0f, seg);
     }
@@ -528,7 +601,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
       float* dst = seg + i * (kRmWarpSamples * 8);
       for (int q = lane; q < kRmWarpSamples * 8; q += 32) dst[q] = dst[q - kRmWarpSamples * 8];
       __syncwarp();
-      rm_euler_step<D, false>(tab, nstage, sm, dst, bias, eta, s0, N, 0, nullptr, nullptr);
+      rm_euler_step<D, false>(tab, one, sm, dst, bias, eta, s0, N, 0, nullptr, nullptr);
     }
     for (int i = kseg - 1; i >= 0; --i) {
       const float* xi = seg + i * (kRmWarpSamples * 8);
@@ -597,6 +670,63 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
   }
 }
 
+// Blocks per tile of a morph: the number (1, 2, 4, 8) with the shortest predicted time.
+// With n blocks together on an SM a stage of 128 features takes stage_us[n]; a
+// launch runs full waves of per_sm blocks an SM and then what is left; adding
+// the blocks' sums up costs a sweep 0.16 + 0.085 cs stages.  The figures are
+// fitted to launches of 2000 to 131,072 samples, M = 1000 and 4096, each with 1,
+// 2, 4 and 8 blocks: the choice is on average 1 % and at worst 9 % slower than the
+// best of the four.  Measured (us, T = 20, M = 4096; 1 / 2 / 4 / 8 blocks): 94
+// tiles 1480 / 1080 / 786 / 840, 157 tiles 2120 / 1499 / 1289 / 1228, 513 tiles
+// 3654 / 3280 / 3275 / 3546, 1024 tiles 6187 / 6367 / 6428 / 6920.
+// An SM holds five blocks of the kernel for one block per tile, four of the others.
+static int rm_cluster(int64_t tiles, int nstage) {
+  static const double stage_us[6] = {0.0, 3.3, 4.7, 6.1, 8.4, 8.5};
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
+                                                 cudaSuccess || sms < 1)
+    sms = 152;
+  int best = 1;
+  double best_t = 0.0;
+  for (int cs = 1; cs <= 8 && cs <= nstage; cs *= 2) {
+    const int per_sm = cs == 1 ? 5 : 4;
+    const int64_t blocks = tiles * cs, wave = (int64_t)sms * per_sm, left = blocks % wave;
+    const double stages = cs == 1 ? (double)nstage : 0.93 * ((nstage + cs - 1) / cs + 0.16 + 0.085 * cs);
+    const double t = ((double)(blocks / wave) * stage_us[per_sm] + stage_us[(left + sms - 1) / sms]) * stages;
+    if (cs == 1 || t < best_t) {
+      best = cs;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
+template <typename Fn, typename... A>
+static cudaError_t rm_launch(Fn fn, int64_t tiles, int cs, size_t smem, cudaStream_t st, A... args) {
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)(tiles * cs));
+  c.blockDim = dim3(kRmWarps * 32);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = cs > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&c, fn, args...);
+}
+// fn: a kernel template over the blocks per tile
+#define PDMP_RM_LAUNCH(cs, tiles, smem, st, KERNEL, ...)                                                     \
+  ((cs) == 8   ? rm_launch(KERNEL(8), tiles, 8, smem, st, __VA_ARGS__)                                       \
+   : (cs) == 4 ? rm_launch(KERNEL(4), tiles, 4, smem, st, __VA_ARGS__)                                       \
+   : (cs) == 2 ? rm_launch(KERNEL(2), tiles, 2, smem, st, __VA_ARGS__)                                       \
+               : rm_launch(KERNEL(1), tiles, 1, smem, st, __VA_ARGS__))
+constexpr size_t kRmShareBytes = (size_t)kRmWarps * kRmWarpSamples * 8 * sizeof(float);   // one array of sums
+
 template <int D>
 static cudaError_t launch_rff_mma(const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, float* xT,
                                   float* ckpt, int k, float* traj, float* steps, void* ws, cudaStream_t st) {
@@ -604,21 +734,20 @@ static cudaError_t launch_rff_mma(const FieldArgs& fa, const float* x0, int64_t 
   const int64_t n_kt = rm_tiles(fa.M);
   k_rff_mma_table<D, false><<<(unsigned)((n_kt * 32 + 255) / 256), 256, 0, st>>>(fa, n_kt, tab);
   const int nstage = (int)(n_kt / kRmStageKT);
-  constexpr size_t smem = rm_smem_bytes();
-  const unsigned blocks = (unsigned)((N + kRmSamples - 1) / kRmSamples);
-  cudaError_t e;
-  if (traj != nullptr) {
-    e = cudaFuncSetAttribute(k_morph_rff_mma<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_morph_rff_mma<D, true><<<blocks, kRmWarps * 32, smem, st>>>(tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k,
-                                                                  traj, steps);
-  } else {
-    e = cudaFuncSetAttribute(k_morph_rff_mma<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_morph_rff_mma<D, false><<<blocks, kRmWarps * 32, smem, st>>>(tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k,
-                                                                   nullptr, nullptr);
-  }
-  return cudaGetLastError();
+  const int64_t tiles = (N + kRmSamples - 1) / kRmSamples;
+  // Checkpoints are where a VJP's replay starts, which runs one block per tile: their
+  // sums are taken the same way, so that each segment ends where the next begins.
+  const int cs = ckpt ? 1 : rm_cluster(tiles, nstage);
+  const size_t smem = rm_smem_bytes() + (cs > 1 ? kRmShareBytes : 0);
+#define PDMP_KERNEL(CS) (k_morph_rff_mma<D, true, CS>)
+  if (traj != nullptr)
+    return PDMP_RM_LAUNCH(cs, tiles, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, traj,
+                          steps);
+#undef PDMP_KERNEL
+#define PDMP_KERNEL(CS) (k_morph_rff_mma<D, false, CS>)
+  return PDMP_RM_LAUNCH(cs, tiles, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, nullptr,
+                        nullptr);
+#undef PDMP_KERNEL
 }
 
 cudaError_t morph_rff_mma(int d, const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, float* xT,
