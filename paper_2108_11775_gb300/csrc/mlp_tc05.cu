@@ -13,14 +13,21 @@
 // The epilogue of a layer reads D from TMEM (thread = sample row, sixteen
 // warps: warps w, w + 4, w + 8 and w + 12 share the TMEM lanes 32 (w % 4) ..
 // + 31 and take 32 columns each), adds the bias, applies SiLU and writes the
-// next A.  (Sixteen warps ran 5 % faster than eight of 64 columns each:
-// 0.438 against 0.462 ms for 2^20 samples.)
+// next A.
 // Three tiles are in flight per CTA: while the epilogue warps run one tile's
 // epilogue the tensor core runs another tile's next layer.  A warp of its own
 // issues the MMAs; the two sides hand tiles over through mbarriers (the
 // issuer's commit to "D ready", the epilogue warps' arrivals to "A ready"),
-// so neither waits at a block barrier (2^20 samples: 0.324 ms against 0.438
-// with block barriers and the MMAs issued by an epilogue thread).
+// so neither waits at a block barrier.
+// What bounds it is the epilogues: 402 sines, cosines and tanh a sample on the
+// special-function unit are 0.37 ms of 2^22 samples' 0.68, the rest is latency
+// of four warps per scheduler.  So the epilogues carry little else (packed
+// FP32 pairs, the bias folded into the halving, one conversion a pair), the
+// encoding is compiled per column group, which makes each feature's octave a
+// constant (before: divisions, selects and a spill; 1.18 ms), the next tile's
+// accumulators are loaded during an epilogue, and a tile's next encoding
+// comes right behind its output.  Tiles are dealt evenly over the SMs: 1024
+// samples take eight SMs instead of three (34 -> 24 us a call).
 //
 // FP32-activation mode (diagnostic): one tile in flight, the activations as
 // three BF16 pieces (three MMA chains over the same weights), the encoding as
@@ -33,6 +40,7 @@
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
+#include "fast_tile.cuh"
 #include "mlp_common.cuh"
 #include "tc05.cuh"
 
@@ -58,7 +66,7 @@ constexpr uint32_t kSbo128 = (kH * 2 / 16) * 128;           // 2048
 
 template <bool EXACT>
 struct Cfg {
-  // tiles in flight: 3 (2^20 samples: 0.311 ms; 2 tiles 0.324, 4 tiles 0.332)
+  // tiles in flight: 3 (2^22 samples: 0.67 ms; 2 tiles 1.01, 4 tiles 0.71)
   static constexpr int kTiles = EXACT ? 1 : 3;
   static constexpr uint32_t kTmemCols = kTiles * kH <= 256 ? 256u : 512u;
   static constexpr int kPieces = EXACT ? 3 : 1;    // BF16 pieces of a hidden activation
@@ -96,13 +104,38 @@ __device__ __forceinline__ float tanh_approx(float x) {
   return y;
 }
 
-// SiLU: z sigma(z) = z (1 + tanh(z / 2)) / 2 on the special-function unit;
-// the FP32-activation mode takes z / (1 + e^-z) with CUDA's expf
-template <bool EXACT>
-__device__ __forceinline__ float silu(float z) {
-  if constexpr (EXACT) return z / (1.0f + expf(-z));
-  const float h = 0.5f * z;
-  return fmaf(h, tanh_approx(h), h);
+// SiLU: z sigma(z) = z (1 + tanh(z / 2)) / 2 on the special-function unit, of a
+// packed pair h = z / 2, as a BF16 pair; the FP32-activation mode takes
+// z / (1 + e^-z) with CUDA's expf
+__device__ __forceinline__ uint32_t silu2(u64 h) {
+  float h0, h1, s0, s1;
+  upk(h, h0, h1);
+  upk(fma2(h, pk(tanh_approx(h0), tanh_approx(h1)), h), s0, s1);
+  return pack2(s0, s1);
+}
+__device__ __forceinline__ float silu_exact(float z) { return z / (1.0f + expf(-z)); }
+
+// Feature pairs [6 G, 6 G + 6) of the encoding of u as two BF16 pieces, into row
+// `row` of a layer-1 A buffer.  With the group a constant, every feature's octave,
+// coordinate and function are, and a sine and a cosine share their angle.
+template <int G>
+__device__ __forceinline__ void encode_pairs(const MlpEncIn& u, unsigned char* dst, int row) {
+  constexpr int np = kEncPad / 2 / kGroups;
+  static_assert(np % 2 == 0, "two pairs a store");
+#pragma unroll
+  for (int i = 0; i < np; i += 2) {
+    uint32_t hi[2], lo[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int f = 2 * (np * G + i + q);
+      const float v0 = mlp_enc_feature<false>(f, u), v1 = mlp_enc_feature<false>(f + 1, u);
+      hi[q] = pack2(v0, v1);
+      lo[q] = pack2(v0 - __uint_as_float(hi[q] << 16), v1 - __uint_as_float(hi[q] & 0xffff0000u));
+    }
+    const int f = 2 * (np * G + i);   // a multiple of 4: 8 bytes within a core-matrix row of 16
+    *reinterpret_cast<uint2*>(dst + tc05::kmajor_offset(row, f, 12, 2)) = make_uint2(hi[0], hi[1]);
+    *reinterpret_cast<uint2*>(dst + tc05::kmajor_offset(row, kEncPad + f, 12, 2)) = make_uint2(lo[0], lo[1]);
+  }
 }
 
 struct MlpTcArgs {
@@ -149,7 +182,8 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
       const uint32_t v = n < 3 ? ((uint32_t)W4[n * kH + k] | ((uint32_t)W4[n * kH + k + 1] << 16)) : 0u;
       *reinterpret_cast<uint32_t*>(sm + C::kOffW4 + tc05::kmajor_offset(n, k, 16, 2)) = v;
     }
-    for (int i = tid; i < 3 * kH + 4; i += kThreads) bias[i] = i < 3 * kH + 3 ? a.b[i] : 0.0f;
+    for (int i = tid; i < 3 * kH + 4; i += kThreads)
+      bias[i] = i < 3 * kH ? (EXACT ? 1.0f : 0.5f) * a.b[i] : (i < 3 * kH + 3 ? a.b[i] : 0.0f);   // hidden: see hidden()
     if (tid == 0) {
       for (int t = 0; t < C::kTiles; ++t) {
         tc05::mbar_init(&bar[t], 1);                    // tile t's MMAs done (commit)
@@ -176,31 +210,27 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
     abort_sh = 1;
   };
   const int64_t tiles = (N + kRows - 1) / kRows;
-  const int64_t groups = (tiles + C::kTiles - 1) / C::kTiles;
+  // the block's tiles, in groups of kTiles (the last of what is left)
+  const int64_t first = tiles * blockIdx.x / gridDim.x, end = tiles * (blockIdx.x + 1) / gridDim.x;
 
   if (warp == kCWarps) {
     // ---------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      uint32_t pa[C::kTiles], pd[C::kTiles];
-      bool pending[C::kTiles];
-#pragma unroll
-      for (int t = 0; t < C::kTiles; ++t) {
-        pa[t] = 0u;
-        pd[t] = 0u;
-        pending[t] = false;
-      }
+      uint32_t pa = 0u, pd = 0u, pending = 0u;   // a bit per tile in flight
       bool ok = true;
-      for (int64_t grp = blockIdx.x; grp < groups && ok; grp += gridDim.x)
+      for (int64_t base = first; base < end && ok; base += C::kTiles) {
+        const int nt = (int)min64(C::kTiles, end - base);
 #pragma unroll 1
         for (int layer = 1; layer <= 4 && ok; ++layer)
 #pragma unroll
           for (int t = 0; t < C::kTiles; ++t) {
-            if (abort_sh || !tc05::mbar_wait(&bar_a[t], pa[t], kWaitClocks)) {
+            if (t >= nt) break;
+            if (abort_sh || !tc05::mbar_wait(&bar_a[t], pa >> t & 1u, kWaitClocks)) {
               fail();
               ok = false;
               break;
             }
-            pa[t] ^= 1u;
+            pa ^= 1u << t;
             tc05::fence_after_sync();
             const uint32_t d = tmem + (uint32_t)(t * kH);
             uint32_t acc = 0u;
@@ -226,29 +256,28 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
                 }
             }
             tc05::commit(&bar_d[t]);
-            if (pending[t]) pd[t] ^= 1u;   // the previous commit of this tile has been waited for by the epilogue
-            pending[t] = true;
+            pd ^= pending & 1u << t;   // the previous commit of this tile has been waited for by the epilogue
+            pending |= 1u << t;
           }
+      }
       // before the tensor memory is freed: this thread's last commit of each tile (bounded)
 #pragma unroll
       for (int t = 0; t < C::kTiles; ++t)
-        if (pending[t]) tc05::mbar_wait(&bar_d[t], pd[t], kWaitClocks);
+        if (pending >> t & 1u) tc05::mbar_wait(&bar_d[t], pd >> t & 1u, kWaitClocks);
     }
   } else {
     // ---------------------------------------------------------- epilogue warps
-    uint32_t pd[C::kTiles];
-#pragma unroll
-    for (int t = 0; t < C::kTiles; ++t) pd[t] = 0u;
+    uint32_t pd = 0u;   // a bit per tile in flight
     // lane 0 waits for the warp (bounded); false after any failure
     auto wait_d = [&](int t) -> bool {
       int ok_ = 1;
       if (lane == 0) {
-        ok_ = !abort_sh && tc05::mbar_wait(&bar_d[t], pd[t], kWaitClocks);
+        ok_ = !abort_sh && tc05::mbar_wait(&bar_d[t], pd >> t & 1u, kWaitClocks);
         if (!ok_) fail();
       }
       __syncwarp();
       ok_ = __shfl_sync(0xffffffffu, ok_, 0);
-      if (ok_) pd[t] ^= 1u;
+      if (ok_) pd ^= 1u << t;
       tc05::fence_after_sync();
       return ok_ != 0;
     };
@@ -260,40 +289,60 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc05::smem_u32(&bar_a[t])) : "memory");
     };
+    const int64_t lim = min64(N, end * kRows);   // the block's own rows (y may be x0)
+    auto load_x = [&](int64_t n, float (&xv)[3]) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) xv[j] = n < lim ? x0[n * 3 + j] : 0.0f;
+    };
     // the encoding of tile t's samples into its layer-1 A buffers: this thread
     // writes K pairs [6 cg, 6 cg + 6) of its row (pairs 0..23)
-    auto encode = [&](int t, int64_t n0) {
-      float xv[3] = {0.0f, 0.0f, 0.0f};
-      const int64_t n = n0 + row;
-      if (n < N)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) xv[j] = x0[n * 3 + j];
+    auto encode = [&](int t, const float (&xv)[3]) {
       MlpEncIn u;
       mlp_enc_prepare(xv, a.lo, a.in_scale, u);
+      if constexpr (!EXACT) {
+        unsigned char* dst = sm + a_buf(t, 0);
+        if (cg == 0) encode_pairs<0>(u, dst, row);
+        else if (cg == 1) encode_pairs<1>(u, dst, row);
+        else if (cg == 2) encode_pairs<2>(u, dst, row);
+        else encode_pairs<3>(u, dst, row);
+        return;
+      }
       constexpr int np = kEncPad / 2 / kGroups;
       static_assert(np * kGroups == kEncPad / 2, "the encoding's K pairs split evenly over the column groups");
 #pragma unroll
       for (int i = 0; i < np; ++i) {
         const int kp = np * cg + i;
         const float v0 = mlp_enc_feature<EXACT>(2 * kp, u), v1 = mlp_enc_feature<EXACT>(2 * kp + 1, u);
-        if constexpr (EXACT) {
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, 2 * kp, 12, 2)) =
-              pack2(piece(v0, 0), piece(v1, 0));
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, kEncPad + 2 * kp, 12, 2)) =
-              pack2(piece(v0, 1), piece(v1, 1));
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 1) + tc05::kmajor_offset(row, 2 * kp, 12, 2)) =
-              pack2(piece(v0, 2), piece(v1, 2));
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 1) + tc05::kmajor_offset(row, kEncPad + 2 * kp, 12, 2)) = 0u;
-        } else {
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, 2 * kp, 12, 2)) =
-              pack2(piece(v0, 0), piece(v1, 0));
-          *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, kEncPad + 2 * kp, 12, 2)) =
-              pack2(piece(v0, 1), piece(v1, 1));
-        }
+        *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, 2 * kp, 12, 2)) =
+            pack2(piece(v0, 0), piece(v1, 0));
+        *reinterpret_cast<uint32_t*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, kEncPad + 2 * kp, 12, 2)) =
+            pack2(piece(v0, 1), piece(v1, 1));
+        *reinterpret_cast<uint32_t*>(sm + a_buf(t, 1) + tc05::kmajor_offset(row, 2 * kp, 12, 2)) =
+            pack2(piece(v0, 2), piece(v1, 2));
+        *reinterpret_cast<uint32_t*>(sm + a_buf(t, 1) + tc05::kmajor_offset(row, kEncPad + 2 * kp, 12, 2)) = 0u;
       }
     };
 
-    // epilogue of a hidden layer of tile t: D (this thread's row, its
+    // BF16 mode: 16 columns from col0 of a hidden layer's epilogue, out of TMEM
+    // already (r).  bl holds half the bias: z / 2 = r / 2 + b / 2 in one rounding, z's.
+    auto hidden16 = [&](int t, const uint32_t (&r)[16], int col0, const float* bl) {
+      const float4* hb = reinterpret_cast<const float4*>(bl + col0);
+      const u64 half = pk(0.5f, 0.5f);
+#pragma unroll
+      for (int kc = 0; kc < 2; ++kc) {
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[8 * kc + i]);
+        const float4 b0 = hb[2 * kc], b1 = hb[2 * kc + 1];
+        uint4 w;
+        w.x = silu2(fma2(pk(v[0], v[1]), half, pk(b0.x, b0.y)));
+        w.y = silu2(fma2(pk(v[2], v[3]), half, pk(b0.z, b0.w)));
+        w.z = silu2(fma2(pk(v[4], v[5]), half, pk(b1.x, b1.y)));
+        w.w = silu2(fma2(pk(v[6], v[7]), half, pk(b1.z, b1.w)));
+        *reinterpret_cast<uint4*>(sm + a_buf(t, 0) + tc05::kmajor_offset(row, col0 + 8 * kc, 16, 2)) = w;
+      }
+    };
+    // FP32-activation mode: epilogue of a hidden layer of tile t: D (this thread's row, its
     // kGroupCols columns) + bias, SiLU, into the next layer's A pieces
     auto hidden = [&](int t, const float* bl) {
 #pragma unroll 1
@@ -302,7 +351,7 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
         float v[32];
         tc05::ld32(taddr_lane + (uint32_t)(t * kH + col0), v);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = silu<EXACT>(v[i] + bl[col0 + i]);
+        for (int i = 0; i < 32; ++i) v[i] = silu_exact(v[i] + bl[col0 + i]);
 #pragma unroll
         for (int p = 0; p < C::kPieces; ++p)
 #pragma unroll
@@ -318,35 +367,108 @@ k_mlp_forward_tc05(MlpTcArgs a, const float* __restrict__ x0, int64_t N, float* 
     };
 
 
-    bool ok = true;
-    for (int64_t grp = blockIdx.x; grp < groups && ok; grp += gridDim.x) {
-      int64_t n0[C::kTiles];
+    // a group's samples are read while the group before runs, and a tile's next
+    // encoding follows its output, while the other tiles' last layers run
+    float xs[C::kTiles][3];
+    auto pick = [&](const float (&v)[C::kTiles][3], int t, float (&x)[3]) {
 #pragma unroll
-      for (int t = 0; t < C::kTiles; ++t) {
-        n0[t] = (grp * C::kTiles + t) * kRows;
-        encode(t, n0[t]);
-        ready(t);
+      for (int j = 0; j < 3; ++j) {
+        x[j] = v[0][j];
+#pragma unroll
+        for (int q = 1; q < C::kTiles; ++q) x[j] = t == q ? v[q][j] : x[j];
+      }
+    };
+#pragma unroll
+    for (int t = 0; t < C::kTiles; ++t) load_x((first + t) * kRows + row, xs[t]);
+#pragma unroll 1
+    for (int t = 0; t < (int)min64(C::kTiles, end - first); ++t) {
+      float x[3];
+      pick(xs, t, x);
+      encode(t, x);
+      ready(t);
+    }
+    const int col0 = kGroupCols * cg;
+    const uint32_t ta = taddr_lane + (uint32_t)col0;
+    bool ok = true;
+    for (int64_t base = first; base < end && ok; base += C::kTiles) {
+      const int nt = (int)min64(C::kTiles, end - base);
+      const int64_t after = end - base - C::kTiles;   // tiles of the groups after this one
+      float xn[C::kTiles][3];
+#pragma unroll
+      for (int t = 0; t < C::kTiles; ++t) load_x((base + C::kTiles + t) * kRows + row, xn[t]);
+      const float* bl = bias;
+      if constexpr (EXACT) {
+#pragma unroll 1
+        for (int layer = 1; layer <= 3; ++layer, bl += kH) {
+          if (!(ok = wait_d(0))) break;
+          hidden(0, bl);
+          ready(0);
+        }
+      } else {
+        // With other tiles in flight, the next epilogue's accumulators come out
+        // of TMEM while this one is computed: half A's once half A is done, half
+        // B's behind half B.  (Waiting for the next tile before this one is
+        // handed over is safe: the next one's MMAs need only its own hand-over
+        // of the layer before.)
+        uint32_t ra[16], rb[16];
+        auto fetch = [&](int t) {
+          tc05::ld16_issue(ta + (uint32_t)(t * kH), ra);
+          tc05::ld16_issue(ta + (uint32_t)(t * kH) + 16u, rb);
+        };
+        if (nt == C::kTiles) {
+          if ((ok = wait_d(0))) fetch(0);
+#pragma unroll 1
+          for (int layer = 1; layer <= 3 && ok; ++layer, bl += kH)
+#pragma unroll
+            for (int t = 0; t < C::kTiles; ++t) {
+              const int next = (t + 1) % C::kTiles;
+              const bool ahead = t + 1 < C::kTiles || layer < 3;
+              const uint32_t tn = ta + (uint32_t)(next * kH);
+              tc05::ld16_wait(ra, rb);
+              hidden16(t, ra, col0, bl);
+              if (ahead && (ok = wait_d(next))) tc05::ld16_issue(tn, ra);
+              if (!ok) break;
+              hidden16(t, rb, col0 + 16, bl);
+              if (ahead) tc05::ld16_issue(tn + 16u, rb);
+              ready(t);
+            }
+        } else {   // the block's last tiles
+#pragma unroll 1
+          for (int layer = 1; layer <= 3 && ok; ++layer, bl += kH)
+#pragma unroll 1
+            for (int t = 0; t < nt; ++t) {
+              if (!(ok = wait_d(t))) break;
+              fetch(t);
+              tc05::ld16_wait(ra, rb);
+              hidden16(t, ra, col0, bl);
+              hidden16(t, rb, col0 + 16, bl);
+              ready(t);
+            }
+        }
       }
 #pragma unroll 1
-      for (int layer = 1; layer <= 3 && ok; ++layer)
-#pragma unroll
-        for (int t = 0; t < C::kTiles; ++t) {
-          if (!(ok = wait_d(t))) break;
-          hidden(t, bias + (layer - 1) * kH);
-          ready(t);
-        }
-#pragma unroll
-      for (int t = 0; t < C::kTiles && ok; ++t) {
+      for (int t = 0; t < nt && ok; ++t) {
         if (!(ok = wait_d(t))) break;
+        float x[3];
         if (cg == 0) {
           float o[16];
           tc05::ld16(taddr_lane + (uint32_t)(t * kH), o);
-          const int64_t n = n0[t] + row;
+          const int64_t n = (base + t) * kRows + row;
+          pick(xs, t, x);
           if (n < N)
 #pragma unroll
-            for (int j = 0; j < 3; ++j) y[n * 3 + j] = fmaf(o[j] + bias[3 * kH + j], a.out_scale[j], x0[n * 3 + j]);
+            for (int j = 0; j < 3; ++j) y[n * 3 + j] = fmaf(o[j] + bias[3 * kH + j], a.out_scale[j], x[j]);
+        }
+        if (t < after) {
+          pick(xn, t, x);
+          encode(t, x);
+          ready(t);
         }
       }
+#pragma unroll
+      for (int t = 0; t < C::kTiles; ++t)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) xs[t][j] = xn[t][j];
     }
   }
   tc05::fence_before_sync();
@@ -374,8 +496,7 @@ cudaError_t launch(const pdmp_mlp* net, const float* x0, int64_t N, float* y, cu
   int dev = 0, sms = 1;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int64_t groups = ((N + kRows - 1) / kRows + C::kTiles - 1) / C::kTiles;
-  const int grid = (int)(groups < sms ? groups : sms);
+  const int grid = (int)min64((N + kRows - 1) / kRows, sms);
   k_mlp_forward_tc05<EXACT><<<grid, kThreads, C::kBytes, st>>>(a, x0, N, y);
   return cudaGetLastError();
 }
