@@ -6,31 +6,25 @@
 // (without it the displacement field, sharp near obstacle boundaries, is out
 // of reach of a small SiLU network).  BF16 weights, FP32 accumulation.
 //
-// Inference runs on the fifth-generation tensor cores (mlp_tc05.cu).  The
-// training kernels here use warp-level MMAs (mma.sync m16n8k16, BF16 x BF16 ->
-// FP32) over the batch: a warp owns 16 samples, and the accumulator fragments
-// of one layer, after bias + SiLU and rounding to BF16, are exactly the A
-// fragments of the next layer, so activations never leave registers.  The
-// 39 -> 128 input layer is FP32 on the CUDA cores.
+// Inference runs on the fifth-generation tensor cores (mlp_tc05.cu), the
+// training step in mlp_train.cu.  The kernels here are the gradient's
+// FP32-activation mode (diagnostic): warp-level MMAs (mma.sync m16n8k16, BF16 x
+// BF16 -> FP32) over the batch, a warp owns 16 samples, and the accumulator
+// fragments of one layer, after bias + SiLU, are exactly the A fragments of the
+// next layer, so activations never leave registers.  The 39 -> 128 input layer
+// is FP32 on the CUDA cores.  Every activation and backward signal is fed to
+// the tensor cores as the sum of three BF16 pieces (hi + mid + lo, which carry
+// 24 bits and more of the FP32 value), so the products are those of FP32
+// activations with the BF16 weights.  The network's arithmetic then matches an
+// FP64 evaluation of the same BF16 weights to FP32 rounding, which separates a
+// fragment-layout fault from BF16 rounding.
 //
-// Training: forward with saved pre-activations, backward through the same
-// fragment layouts (dA = dZ W on the tensor cores with transposed weight
-// copies), then the weight and bias gradients of every layer as one more
-// tensor-core contraction per layer, [dW | db] = dZ^T [a | 1] over the batch
-// (BF16 operands staged transposed in shared memory, FP32 accumulation;
-// blocks of 64 samples write partial sums that a second kernel adds in a
-// fixed order), and Adam on FP32 master weights that rewrites the BF16 copies.
-//
-// FP32-activation mode (diagnostic): the same kernels and fragment layouts
-// with every activation and backward signal fed to the tensor cores as the
-// sum of three BF16 pieces (hi + mid + lo, which carry 24 bits and more of
-// the FP32 value), so the products are those of FP32 activations with the
-// BF16 weights.  The network's arithmetic then matches an FP64 evaluation of
-// the same BF16 weights to FP32 rounding, which separates a fragment-layout
-// fault from BF16 rounding.
-#include <cuda_bf16.h>
-
-#include "kernels.cuh"
+// Forward with saved pre-activations, backward through the same fragment
+// layouts (dA = dZ W on the tensor cores with transposed weight copies), then
+// the weight and bias gradients of every layer as one more tensor-core
+// contraction per layer, [dW | db] = dZ^T [a | 1] over the batch (operands staged
+// transposed in shared memory, FP32 accumulation; blocks of 64 samples write
+// partial sums that a second kernel adds in a fixed order).
 #include "mlp_common.cuh"
 
 namespace pdmp {
@@ -40,39 +34,6 @@ constexpr int kFreq = 6;         // octaves of the input encoding
 constexpr int kEnc = 3 + 6 * kFreq;   // encoded input width (39)
 constexpr int kRowU32 = 68;      // padded smem row: 136 bf16 = 68 words (conflict-free fragment loads)
 constexpr int kMlpWarps = 4;
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-__device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-
-__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ float silu_f(float z) { return z / (1.0f + __expf(-z)); }
-__device__ __forceinline__ float silu_grad_f(float z) {
-  const float s = 1.0f / (1.0f + __expf(-z));
-  return s * (1.0f + z * (1.0f - s));
-}
-
-// Device copy of the network (all pointers device; bf16 as raw uint16).
-struct MlpArgs {
-  const uint16_t* W1;   // 128 x 39
-  const uint16_t* W2;   // 128 x 128  [out][in]
-  const uint16_t* W3;   // 128 x 128
-  const uint16_t* W4;   // 3 x 128
-  const uint16_t* W2t;  // 128 x 128  [in][out] (backward)
-  const uint16_t* W3t;  // 128 x 128
-  const float *b1, *b2, *b3, *b4;
-  float lo[3], in_scale[3], out_scale[3];
-};
 
 // shared-memory image of the weights
 struct MlpSmem {
@@ -160,40 +121,30 @@ __device__ __forceinline__ void gemm_128_acc(const uint32_t (&af)[8][4], const u
     }
 }
 
-// v <- v W^T (v: a warp's 16 rows of activations in C-fragment layout).
-// EXACT: v enters as three BF16 pieces (FP32-activation mode).
-template <bool EXACT>
+// v <- v W^T (v: a warp's 16 rows of activations in C-fragment layout), v as
+// three BF16 pieces
 __device__ __forceinline__ void dense_128(float (&v)[16][4], const uint32_t* W, int g, int t) {
-  if constexpr (EXACT) {
-    float h[16][4];
+  float h[16][4];
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
+  for (int j = 0; j < 16; ++j)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        h[j][q] = v[j][q];
-        v[j][q] = 0.0f;
-      }
-#pragma unroll 1
-    for (int p = 0; p < 3; ++p) {
-      uint32_t af[8][4];
-      to_afrag(h, p, af);
-      gemm_128_acc(af, W, g, t, v);
+    for (int q = 0; q < 4; ++q) {
+      h[j][q] = v[j][q];
+      v[j][q] = 0.0f;
     }
-  } else {
+#pragma unroll 1
+  for (int p = 0; p < 3; ++p) {
     uint32_t af[8][4];
-    to_afrag(v, 0, af);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j][0] = v[j][1] = v[j][2] = v[j][3] = 0.0f;
+    to_afrag(h, p, af);
     gemm_128_acc(af, W, g, t, v);
   }
 }
 
 // o (one n8 tile: columns 2t, 2t + 1 of rows g, g + 8) = v W4^T
-template <bool EXACT>
 __device__ __forceinline__ void dense_out(const float (&v)[16][4], const uint32_t* W4, int g, int t, float (&o)[4]) {
   o[0] = o[1] = o[2] = o[3] = 0.0f;
 #pragma unroll 1
-  for (int p = 0; p < (EXACT ? 3 : 1); ++p) {
+  for (int p = 0; p < 3; ++p) {
     uint32_t af[8][4];
     to_afrag(v, p, af);
 #pragma unroll
@@ -204,15 +155,13 @@ __device__ __forceinline__ void dense_out(const float (&v)[16][4], const uint32_
   }
 }
 
-// the Fourier encoding of x's normalised coordinates (mlp_common.cuh); the
-// training kernels take sin / cos on the special-function unit, the
-// FP32-activation mode CUDA's sinf / cosf
-template <bool EXACT>
+// the Fourier encoding of x's normalised coordinates (mlp_common.cuh) with
+// CUDA's sinf / cosf
 __device__ __forceinline__ void encode(const MlpArgs& a, const float* x, float* e) {
   MlpEncIn in;
   mlp_enc_prepare(x, a.lo, a.in_scale, in);
 #pragma unroll
-  for (int f = 0; f < kEnc; ++f) e[f] = mlp_enc_feature<EXACT>(f, in);
+  for (int f = 0; f < kEnc; ++f) e[f] = mlp_enc_feature<true>(f, in);
 }
 
 // input layer (FP32): acc[j] = W1 enc for rows g, g + 8 of the warp's tile
@@ -243,7 +192,6 @@ __device__ __forceinline__ void input_layer(const MlpSmem* s, const float* e0, c
 // input u (B x 3) and dY = d loss / d output (B x 3) for the MSE loss against
 // target (x_T - x_0) / out_scale; loss_rows[tile * 16 + r] gets row r's
 // squared error (summed in a fixed order later).
-template <bool EXACT>
 __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_forward(MlpArgs a, const float* __restrict__ x0,
                                                                        const float* __restrict__ xT, int B,
                                                                        float* __restrict__ Z,   // 3 x B x 128
@@ -267,8 +215,8 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_forward(MlpArgs a,
 #pragma unroll
       for (int i = 0; i < 3; ++i) x_1[i] = x0[r1 * 3 + i];
     float e0[kEnc], e1[kEnc];
-    encode<EXACT>(a, x_0, e0);
-    encode<EXACT>(a, x_1, e1);
+    encode(a, x_0, e0);
+    encode(a, x_1, e1);
     if (t == 0) {
       if (r0 < B)
 #pragma unroll
@@ -280,12 +228,12 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_forward(MlpArgs a,
     float acc[16][4];
     input_layer(s, e0, e1, t, acc);
     bias_silu(acc, s->b1, t, Z, r0, r1, B);
-    dense_128<EXACT>(acc, s->W2, g, t);
+    dense_128(acc, s->W2, g, t);
     bias_silu(acc, s->b2, t, Z + (size_t)B * kH, r0, r1, B);
-    dense_128<EXACT>(acc, s->W3, g, t);
+    dense_128(acc, s->W3, g, t);
     bias_silu(acc, s->b3, t, Z + (size_t)2 * B * kH, r0, r1, B);
     float o[4];
-    dense_out<EXACT>(acc, s->W4, g, t, o);
+    dense_out(acc, s->W4, g, t, o);
     float q0 = 0.0f, q1 = 0.0f;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -317,7 +265,6 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_forward(MlpArgs a,
 
 // Backward through the activations: dZ3 = (dY W4) * silu'(z3), dZ2 = (dZ3 W3) * silu'(z2),
 // dZ1 = (dZ2 W2) * silu'(z1), into dZ (3 x B x 128); Z holds the pre-activations.
-template <bool EXACT>
 __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_backward(MlpArgs a, int B, const float* __restrict__ dY,
                                                                         const float* __restrict__ Z,
                                                                         float* __restrict__ dZ) {
@@ -372,7 +319,7 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_backward(MlpArgs a
       }
       if (l == 0) break;
       // dA_{l-1} = dZ_l W_l: B operand (k = out, n = in) from the transposed image W_l^T[in][out]
-      dense_128<EXACT>(acc, l == 2 ? s->W3 : s->W2, g, t);
+      dense_128(acc, l == 2 ? s->W3 : s->W2, g, t);
     }
   }
 }
@@ -384,15 +331,14 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_train_backward(MlpArgs a
 // operands are staged transposed (rows = output / input unit, 32 BF16 pairs of
 // samples per row) so that fragments are 32-bit loads, and the block writes its
 // partial sums to part[blockIdx.x] (weights then biases, the layout of gW, gb).
-// EXACT: both operands as three BF16 pieces, the six products of pieces whose
+// Both operands as three BF16 pieces, the six products of pieces whose
 // orders add up to at most 2.
 constexpr int kGradKC = 64;                         // samples per block
 constexpr int kGradRow = kGradKC / 2 + 4;           // u32 per staged row (36: conflict-free fragment loads)
 constexpr int kGradRowsA = 128, kGradRowsB = 136;   // output units; input units + the ones row, padded
 
-template <bool EXACT>
 constexpr size_t grad_smem_bytes() {
-  return sizeof(uint32_t) * (EXACT ? 3 : 1) * (kGradRowsA + kGradRowsB) * kGradRow;
+  return sizeof(uint32_t) * 3 * (kGradRowsA + kGradRowsB) * kGradRow;
 }
 
 __device__ __forceinline__ size_t layer_woff(int l) {
@@ -414,7 +360,7 @@ __device__ __forceinline__ void stage_t(uint32_t* dst, int rows, int b0, int B, 
 }
 
 // one warp: MTW m tiles from mt0 x NTW n tiles nt0, nt0 + NS, ... (< NT) of C = A^T-staged x B^T-staged
-template <bool EXACT, int MTW, int NTW, int NS, int NT>
+template <int MTW, int NTW, int NS, int NT>
 __device__ __forceinline__ void grad_tiles(const uint32_t* sA, int rowsA, const uint32_t* sB, int rowsB, int mt0,
                                            int nt0, int O, int I, size_t woff, size_t boff, float* __restrict__ part) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -424,7 +370,7 @@ __device__ __forceinline__ void grad_tiles(const uint32_t* sA, int rowsA, const 
 #pragma unroll
     for (int j = 0; j < NTW; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.0f;
 #pragma unroll 1
-  for (int pp = 0; pp < (EXACT ? 6 : 1); ++pp) {
+  for (int pp = 0; pp < 6; ++pp) {
     // piece pairs (pa, pb) with pa + pb <= 2
     const int pa = pp < 3 ? 0 : (pp < 5 ? 1 : 2), pb = pp < 3 ? pp : (pp < 5 ? pp - 3 : 0);
     const uint32_t* A = sA + (size_t)pa * rowsA * kGradRow;
@@ -469,12 +415,11 @@ __device__ __forceinline__ void grad_tiles(const uint32_t* sA, int rowsA, const 
     }
 }
 
-template <bool EXACT>
 __global__ void __launch_bounds__(128, 1) k_mlp_weight_grads(int B, const float* __restrict__ U,
                                                              const float* __restrict__ Zf, const float* __restrict__ dZ,
                                                              const float* __restrict__ dY, float* __restrict__ part) {
   extern __shared__ __align__(16) uint32_t gsm[];
-  constexpr int P = EXACT ? 3 : 1;
+  constexpr int P = 3;
   const int layer = blockIdx.y, b0 = blockIdx.x * kGradKC, warp = threadIdx.x >> 5;
   const int I = layer == 0 ? kEnc : kH, O = layer == 3 ? 3 : kH;
   const int rowsA = layer == 3 ? 16 : kGradRowsA, rowsB = layer == 0 ? 40 : kGradRowsB;
@@ -494,73 +439,11 @@ __global__ void __launch_bounds__(128, 1) k_mlp_weight_grads(int B, const float*
   __syncthreads();
   const size_t woff = layer_woff(layer), boff = (size_t)layer * kH;
   if (layer == 0)
-    grad_tiles<EXACT, 2, 5, 1, 5>(sA, rowsA, sB, rowsB, 2 * warp, 0, O, I, woff, boff, out);
+    grad_tiles<2, 5, 1, 5>(sA, rowsA, sB, rowsB, 2 * warp, 0, O, I, woff, boff, out);
   else if (layer < 3)
-    grad_tiles<EXACT, 2, 17, 1, 17>(sA, rowsA, sB, rowsB, 2 * warp, 0, O, I, woff, boff, out);
+    grad_tiles<2, 17, 1, 17>(sA, rowsA, sB, rowsB, 2 * warp, 0, O, I, woff, boff, out);
   else
-    grad_tiles<EXACT, 1, 5, 4, 17>(sA, rowsA, sB, rowsB, 0, warp, O, I, woff, boff, out);
-}
-
-// gW, gb = the blocks' partial sums added in block order
-__global__ void k_mlp_grad_sum(const float* __restrict__ part, int nparts, float* __restrict__ gW,
-                               float* __restrict__ gb) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kMlpNW + kMlpNB) return;
-  float acc = 0.0f;
-  for (int c = 0; c < nparts; ++c) acc += part[(size_t)c * (kMlpNW + kMlpNB) + i];
-  if (i < kMlpNW) gW[i] = acc;
-  else gb[i - kMlpNW] = acc;
-}
-
-// Adam on FP32 masters; rewrites the BF16 copies (and the transposed copies of W2, W3)
-__global__ void k_mlp_adam(int64_t nW, int64_t nb, float* __restrict__ W, float* __restrict__ b,
-                           const float* __restrict__ gW, const float* __restrict__ gb, float* __restrict__ mW,
-                           float* __restrict__ vW, float* __restrict__ mb, float* __restrict__ vb, float lr, float beta1,
-                           float beta2, float eps, float c1, float c2, uint16_t* __restrict__ Wbf,
-                           uint16_t* __restrict__ W2t, uint16_t* __restrict__ W3t) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nW) {
-    const float gr = gW[i];
-    const float m = beta1 * mW[i] + (1.0f - beta1) * gr;
-    const float v = beta2 * vW[i] + (1.0f - beta2) * gr * gr;
-    mW[i] = m;
-    vW[i] = v;
-    const float w = W[i] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-    W[i] = w;
-    __nv_bfloat16 wb = __float2bfloat16_rn(w);
-    const uint16_t bits = *reinterpret_cast<uint16_t*>(&wb);
-    Wbf[i] = bits;
-    const int64_t o2 = (int64_t)kEnc * kH, o3 = o2 + kH * kH;
-    if (i >= o2 && i < o3) {
-      const int64_t r = (i - o2) / kH, c = (i - o2) % kH;
-      W2t[c * kH + r] = bits;
-    } else if (i >= o3 && i < o3 + kH * kH) {
-      const int64_t r = (i - o3) / kH, c = (i - o3) % kH;
-      W3t[c * kH + r] = bits;
-    }
-  } else if (i < nW + nb) {
-    const int64_t k = i - nW;
-    const float gr = gb[k];
-    const float m = beta1 * mb[k] + (1.0f - beta1) * gr;
-    const float v = beta2 * vb[k] + (1.0f - beta2) * gr * gr;
-    mb[k] = m;
-    vb[k] = v;
-    b[k] = b[k] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-  }
-}
-
-// fixed-order sum of the per-row squared errors -> mean loss
-__global__ void __launch_bounds__(1024) k_mlp_loss(const float* __restrict__ err, int B, float* __restrict__ loss) {
-  __shared__ double sh[1024];
-  double a = 0.0;
-  for (int i = threadIdx.x; i < B; i += blockDim.x) a += err[i];
-  sh[threadIdx.x] = a;
-  __syncthreads();
-  for (int o = 512; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *loss = (float)(sh[0] / (3.0 * B));
+    grad_tiles<1, 5, 4, 17>(sA, rowsA, sB, rowsB, 0, warp, O, I, woff, boff, out);
 }
 
 // BF16 copies of the FP32 masters (and the transposes of W2, W3)
@@ -622,70 +505,80 @@ cudaError_t mlp_forward(const pdmp_mlp* net, const float* x0, int64_t N, float* 
 
 static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
-static int grad_parts(int B) { return (B + kGradKC - 1) / kGradKC; }
+// The FP32-activation mode's buffers.  The training step keeps activations in
+// shared memory and needs its errors and parts only (train_ws); one size, this
+// mode's, serves both.
+struct TrainWs {
+  float *Z, *dZ, *U, *dY, *err, *part;
+  size_t bytes;
+};
 
-size_t mlp_train_workspace(int B) {
-  return 2 * al256(sizeof(float) * 3 * (size_t)B * kH) + al256(sizeof(float) * kEnc * (size_t)B) +
-         2 * al256(sizeof(float) * 3 * (size_t)B) + al256(sizeof(float) * kMlpNW) + al256(sizeof(float) * kMlpNB) +
-         al256(sizeof(float) * (size_t)grad_parts(B) * (kMlpNW + kMlpNB));
+static TrainWs train_layout(void* ws, int B) {
+  TrainWs w;
+  char* p = (char*)ws;
+  auto take = [&](size_t n) {
+    float* q = (float*)p;
+    p += al256(sizeof(float) * n);
+    return q;
+  };
+  w.Z = take(3 * (size_t)B * kH);
+  w.dZ = take(3 * (size_t)B * kH);
+  w.U = take(kEnc * (size_t)B);
+  w.dY = take(3 * (size_t)B);
+  w.err = take(3 * (size_t)B);
+  take(kMlpNW);
+  take(kMlpNB);
+  w.part = take((size_t)mlp_grad_parts(B) * (kMlpNW + kMlpNB));
+  w.bytes = (size_t)(p - (char*)ws);
+  return w;
 }
 
-template <bool EXACT>
-static cudaError_t launch_gradient(const pdmp_mlp* net, const float* x0, const float* xT, int B, float* loss,
-                                   float* gW, float* gb, char* p, cudaStream_t st) {
-  auto take = [&](size_t b) { char* q = p; p += al256(b); return q; };
-  float* Z = (float*)take(sizeof(float) * 3 * (size_t)B * kH);
-  float* dZ = (float*)take(sizeof(float) * 3 * (size_t)B * kH);
-  float* U = (float*)take(sizeof(float) * kEnc * (size_t)B);
-  float* dY = (float*)take(sizeof(float) * 3 * (size_t)B);
-  float* err = (float*)take(sizeof(float) * 3 * (size_t)B);
-  take(sizeof(float) * kMlpNW);   // gW, gb of the training step
-  take(sizeof(float) * kMlpNB);
-  float* part = (float*)take(sizeof(float) * (size_t)grad_parts(B) * (kMlpNW + kMlpNB));
-  const MlpArgs a = mlp_args(net);
+// the training step's: its parts lie kMlpTrainPart apart, 29 floats more than the
+// FP32 mode's, and the 810 floats a sample (and one more part) that it does
+// without leave room for them
+static TrainWs train_ws(void* ws, int B) {
+  TrainWs w{};
+  w.err = (float*)ws;
+  w.part = (float*)((char*)ws + al256(sizeof(float) * (size_t)B));
+  return w;
+}
+
+size_t mlp_train_workspace(int B) { return train_layout(nullptr, B).bytes; }
+
+static cudaError_t partials_fp32(const MlpArgs& a, const float* x0, const float* xT, int B, const TrainWs& w,
+                                 cudaStream_t st) {
   const size_t smem = sizeof(MlpSmem);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_mlp_train_forward<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+  if ((e = cudaFuncSetAttribute(k_mlp_train_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_mlp_train_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
     return e;
-  if ((e = cudaFuncSetAttribute(k_mlp_train_backward<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-    return e;
-  constexpr size_t gsmem = grad_smem_bytes<EXACT>();
-  if ((e = cudaFuncSetAttribute(k_mlp_weight_grads<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem)))
-    return e;
+  constexpr size_t gsmem = grad_smem_bytes();
+  if ((e = cudaFuncSetAttribute(k_mlp_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem))) return e;
   const int64_t tiles = (B + 15) / 16;
-  const int gf = mlp_grid(tiles, (const void*)k_mlp_train_forward<EXACT>);
-  k_mlp_train_forward<EXACT><<<gf, 32 * kMlpWarps, smem, st>>>(a, x0, xT, B, Z, U, dY, err);
-  if (loss) k_mlp_loss<<<1, 1024, 0, st>>>(err, B, loss);
-  const int gbk = mlp_grid(tiles, (const void*)k_mlp_train_backward<EXACT>);
-  k_mlp_train_backward<EXACT><<<gbk, 32 * kMlpWarps, smem, st>>>(a, B, dY, Z, dZ);
-  k_mlp_weight_grads<EXACT><<<dim3((unsigned)grad_parts(B), 4), 128, gsmem, st>>>(B, U, Z, dZ, dY, part);
-  k_mlp_grad_sum<<<(unsigned)((kMlpNW + kMlpNB + 255) / 256), 256, 0, st>>>(part, grad_parts(B), gW, gb);
+  const int gf = mlp_grid(tiles, (const void*)k_mlp_train_forward);
+  k_mlp_train_forward<<<gf, 32 * kMlpWarps, smem, st>>>(a, x0, xT, B, w.Z, w.U, w.dY, w.err);
+  const int gbk = mlp_grid(tiles, (const void*)k_mlp_train_backward);
+  k_mlp_train_backward<<<gbk, 32 * kMlpWarps, smem, st>>>(a, B, w.dY, w.Z, w.dZ);
+  k_mlp_weight_grads<<<dim3((unsigned)mlp_grad_parts(B), 4), 128, gsmem, st>>>(B, w.U, w.Z, w.dZ, w.dY, w.part);
   return cudaGetLastError();
 }
 
 cudaError_t mlp_gradient(const pdmp_mlp* net, const float* x0, const float* xT, int B, bool fp32_act, float* loss,
                          float* gW, float* gb, void* ws, cudaStream_t st) {
-  return fp32_act ? launch_gradient<true>(net, x0, xT, B, loss, gW, gb, (char*)ws, st)
-                  : launch_gradient<false>(net, x0, xT, B, loss, gW, gb, (char*)ws, st);
+  const MlpArgs a = mlp_args(net);
+  const TrainWs w = fp32_act ? train_layout(ws, B) : train_ws(ws, B);
+  const cudaError_t e = fp32_act ? partials_fp32(a, x0, xT, B, w, st) : mlp_train_partials(a, x0, xT, B, w.err, w.part, st);
+  if (e != cudaSuccess) return e;
+  return mlp_sum_partials(w.part, mlp_grad_parts(B), fp32_act ? (int)(kMlpNW + kMlpNB) : kMlpTrainPart, gW, gb, w.err,
+                          B, loss, st);
 }
 
 cudaError_t mlp_train_step(const pdmp_mlp* net, const float* x0, const float* xT, int B, float lr, float beta1,
                            float beta2, float eps, int step, float* loss, void* ws, cudaStream_t st) {
-  char* p = (char*)ws + 2 * al256(sizeof(float) * 3 * (size_t)B * kH) + al256(sizeof(float) * kEnc * (size_t)B) +
-            2 * al256(sizeof(float) * 3 * (size_t)B);
-  float* gW = (float*)p;
-  float* gb = (float*)(p + al256(sizeof(float) * kMlpNW));
-  cudaError_t e = launch_gradient<false>(net, x0, xT, B, loss, gW, gb, (char*)ws, st);
+  const TrainWs w = train_ws(ws, B);
+  const cudaError_t e = mlp_train_partials(mlp_args(net), x0, xT, B, w.err, w.part, st);
   if (e != cudaSuccess) return e;
-  float* mW = net->adam;
-  float* vW = net->adam + kMlpNW;
-  float* mb = net->adam + 2 * kMlpNW;
-  float* vb = net->adam + 2 * kMlpNW + kMlpNB;
-  const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
-  k_mlp_adam<<<(unsigned)((kMlpNW + kMlpNB + 255) / 256), 256, 0, st>>>(
-      kMlpNW, kMlpNB, net->W, net->b, gW, gb, mW, vW, mb, vb, lr, beta1, beta2, eps, c1, c2, net->W_bf16,
-      net->Wt_bf16, net->Wt_bf16 + kH * kH);
-  return cudaGetLastError();
+  return mlp_adam_step(net, w.part, mlp_grad_parts(B), lr, beta1, beta2, eps, step, w.err, B, loss, st);
 }
 
 }  // namespace pdmp
