@@ -209,10 +209,11 @@ __device__ __forceinline__ u64 rm_turns_to_rad(u64 tau) {
 }
 
 // A fragments (hi, lo) of the warp's 32 rows of a [32][8] state array.
-__device__ __forceinline__ void rm_frags(const float* xs, int g, int t, uint32_t (&ah)[kRmRows][4],
-                                         uint32_t (&al)[kRmRows][4]) {
+template <int R>
+__device__ __forceinline__ void rm_frags(const float* xs, int g, int t, uint32_t (&ah)[R][4],
+                                         uint32_t (&al)[R][4]) {
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r) {
+  for (int r = 0; r < R; ++r) {
     const float* xr = xs + r * 16 * 8;
     const float v[4] = {xr[g * 8 + t], xr[(g + 8) * 8 + t], xr[g * 8 + t + 4], xr[(g + 8) * 8 + t + 4]};
 #pragma unroll
@@ -267,14 +268,14 @@ __device__ __forceinline__ void rm_leave(RmShare& sh) {   // no block leaves whi
 // sum_m cos(theta_m) (omega_m . v / 2 pi) (-w_m omega_m) = (Hess s) v / 2 pi).
 // Block-wide: every warp of the block makes the same sequence of passes.  tab
 // and nstage: the stages of this block (all of them without a cluster).
-template <bool HVP>
+template <bool HVP, int R>
 __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nstage, float* sm,
-                                         const uint32_t (&ah)[kRmRows][4], const uint32_t (&al)[kRmRows][4],
-                                         const uint32_t (&vh)[kRmRows][4], const uint32_t (&vl)[kRmRows][4],
-                                         u64 (&S)[kRmRows][2], float (&G)[kRmRows][4], float (&P)[kRmRows][4]) {
+                                         const uint32_t (&ah)[R][4], const uint32_t (&al)[R][4],
+                                         const uint32_t (&vh)[R][4], const uint32_t (&vl)[R][4],
+                                         u64 (&S)[R][2], float (&G)[R][4], float (&P)[R][4]) {
   const int lane = threadIdx.x & 31, t = lane & 3;
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r) {
+  for (int r = 0; r < R; ++r) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) G[r][q] = P[r][q] = 0.0f;
     S[r][0] = S[r][1] = 0ull;
@@ -298,7 +299,7 @@ __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nsta
       const uint32_t bgh0 = __float_as_uint(bg.x), bgh1 = __float_as_uint(bg.y);
       const uint32_t bgl0 = __float_as_uint(bg.z), bgl1 = __float_as_uint(bg.w);
 #pragma unroll
-      for (int r = 0; r < kRmRows; ++r) {
+      for (int r = 0; r < R; ++r) {
         float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         mma_tf32(d, al[r][0], al[r][1], al[r][2], al[r][3], bth0, bth1);
         mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], btl0, btl1);
@@ -358,7 +359,8 @@ __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nsta
 }
 
 // the logit of rows g (hh = 0) and g + 8 (hh = 1) of row tile r: the quad's partial sums
-__device__ __forceinline__ float rm_logit(const u64 (&S)[kRmRows][2], int r, int hh) {
+template <int R>
+__device__ __forceinline__ float rm_logit(const u64 (&S)[R][2], int r, int hh) {
   float sa, sb;
   upk(S[r][hh], sa, sb);
   float s = sa + sb;
@@ -369,25 +371,25 @@ __device__ __forceinline__ float rm_logit(const u64 (&S)[kRmRows][2], int r, int
 
 // The totals over the cluster's blocks: s (without the bias) of rows r * 16 + g +
 // 8 hh, and G.
-template <int CS>
-__device__ __forceinline__ void rm_combine(RmShare& sh, const u64 (&S)[kRmRows][2], float (&s)[kRmRows][2],
-                                           float (&G)[kRmRows][4]) {
+template <int CS, int R>
+__device__ __forceinline__ void rm_combine(RmShare& sh, const u64 (&S)[R][2], float (&s)[R][2],
+                                           float (&G)[R][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) s[r][hh] = rm_logit(S, r, hh);
-  float* ex = sh.ex + (threadIdx.x >> 5) * (kRmWarpSamples * 8);
+  float* ex = sh.ex + (threadIdx.x >> 5) * ((R * 16) * 8);
   if (sh.pending) cluster_wait();
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh)
       *reinterpret_cast<float2*>(ex + (r * 16 + g + 8 * hh) * 8 + 2 * t) =
           make_float2(G[r][2 * hh], t == 3 ? s[r][hh] : G[r][2 * hh + 1]);
   cluster_barrier();
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
       const float* e = ex + (r * 16 + g + 8 * hh) * 8 + 2 * t;
@@ -405,22 +407,22 @@ __device__ __forceinline__ void rm_combine(RmShare& sh, const u64 (&S)[kRmRows][
   sh.pending = true;
 }
 
-// One Euler step of the warp's 32 samples held in xs ([32][8], column 7 = 1).
-template <int D, bool TRACE, int CS = 1>
+// One Euler step of the warp's 16 R samples held in xs ([16 R][8], column 7 = 1).
+template <int D, bool TRACE, int CS, int R>
 __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, RmShare& sh, float* sm, float* xs,
                                               float bias, float eta, int64_t s0, int64_t N, int step,
                                               float* __restrict__ traj, float* __restrict__ steps) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  uint32_t ah[kRmRows][4], al[kRmRows][4];
+  uint32_t ah[R][4], al[R][4];
   rm_frags(xs, g, t, ah, al);
-  float G[kRmRows][4], P[kRmRows][4];
-  u64 S[kRmRows][2];
+  float G[R][4], P[R][4];
+  u64 S[R][2];
   rm_sweep<false>(CS == 1 ? tab : tab + (size_t)sh.st0 * kRmStageFloats, CS == 1 ? sh.st1 : sh.st1 - sh.st0, sm, ah,
                   al, ah, al, S, G, P);
-  float s[kRmRows][2];
-  if (CS > 1) rm_combine<CS>(sh, S, s, G);
+  float s[R][2];
+  if constexpr (CS > 1) rm_combine<CS>(sh, S, s, G);
 #pragma unroll
-  for (int r = 0; r < kRmRows; ++r) {
+  for (int r = 0; r < R; ++r) {
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
       float d1, d2;
@@ -445,12 +447,12 @@ __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, RmS
   __syncwarp();
 }
 
-// rows [s0, s0 + 32) of an N x D array into xs ([32][8]; column 7 = col7)
-template <int D>
+// rows [s0, s0 + 16 R) of an N x D array into xs ([16 R][8]; column 7 = col7)
+template <int D, int R = kRmRows>
 __device__ __forceinline__ void rm_load_rows(const float* __restrict__ src, int64_t s0, int64_t N, float col7,
                                              float* xs) {
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i < kRmWarpSamples * 8; i += 32) {
+  for (int i = lane; i < (R * 16) * 8; i += 32) {
     const int r = i >> 3, j = i & 7;
     const int64_t n = s0 + r;
     xs[i] = j < D ? (n < N ? src[n * D + j] : 0.0f) : (j == 7 ? col7 : 0.0f);
@@ -458,37 +460,60 @@ __device__ __forceinline__ void rm_load_rows(const float* __restrict__ src, int6
   __syncwarp();
 }
 
-template <int D>
+template <int D, int R = kRmRows>
 __device__ __forceinline__ void rm_store_rows(const float* xs, int64_t s0, int64_t N, float* __restrict__ dst) {
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i < kRmWarpSamples * D; i += 32) {
+  for (int i = lane; i < (R * 16) * D; i += 32) {
     const int r = i / D, j = i % D;
     if (s0 + r < N) dst[(s0 + r) * D + j] = xs[r * 8 + j];
   }
+}
+
+// How a launch deals its samples out to blocks (one block a tile): the first n2
+// blocks take whole tiles of 128 samples, the others halves of 64 (one row tile
+// a warp).  Every sample's sums are the same either way.
+struct RmDeal {
+  unsigned n2, blocks;
+};
+__device__ __forceinline__ int64_t rm_first(unsigned b, unsigned n2) {
+  return b < n2 ? (int64_t)b * kRmSamples : (int64_t)n2 * kRmSamples + (int64_t)(b - n2) * (kRmSamples / 2);
+}
+
+template <int D, bool TRACE, int CS, int R>
+__device__ __forceinline__ void rm_morph_block(float* sm, const float* __restrict__ tab, int nstage, float bias,
+                                               const float* __restrict__ x0, int64_t first, int64_t N, int T, float eta,
+                                               float* __restrict__ xT, float* __restrict__ ckpt, int kck,
+                                               float* __restrict__ traj, float* __restrict__ steps) {
+  const int warp = threadIdx.x >> 5;
+  float* xs = sm + 2 * kRmStageFloats + warp * (R * 16 * 8);   // [16 R samples][8]: x, 0 .., 1
+  RmShare sh = rm_share(CS, nstage, sm + 2 * kRmStageFloats + kRmWarps * (R * 16 * 8));
+  const int64_t s0 = first + warp * (R * 16);
+  rm_load_rows<D, R>(x0, s0, N, 1.0f, xs);
+  for (int step = 0; step < T; ++step) {
+    rm_euler_step<D, TRACE, CS, R>(tab, sh, sm, xs, bias, eta, s0, N, step, traj, steps);
+    if (ckpt != nullptr && (step + 1) % kck == 0 && sh.crank == 0)
+      rm_store_rows<D, R>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
+  }
+  rm_leave<CS>(sh);
+  if (sh.crank > 0) return;
+  if (xT) rm_store_rows<D, R>(xs, s0, N, xT);
+  if (TRACE) rm_store_rows<D, R>(xs, s0, N, traj + (int64_t)T * N * D);
 }
 
 template <int D, bool TRACE, int CS>
 __global__ void __launch_bounds__(kRmWarps * 32, 4)
 k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
                 float eta, float* __restrict__ xT, float* __restrict__ ckpt, int kck, float* __restrict__ traj,
-                float* __restrict__ steps) {
+                float* __restrict__ steps, unsigned n2) {
   static_assert(D >= 1 && D <= 7, "dimensions and the phase share the 8 k slots");
   extern __shared__ __align__(16) float sm[];
   rm_stage_init();
-  const int warp = threadIdx.x >> 5;
-  float* xs = sm + 2 * kRmStageFloats + warp * (kRmWarpSamples * 8);   // [32 samples][8]: x, 0 .., 1
-  RmShare sh = rm_share(CS, nstage, sm + 2 * kRmStageFloats + kRmWarps * (kRmWarpSamples * 8));
-  const int64_t s0 = (int64_t)(blockIdx.x / CS) * kRmSamples + warp * kRmWarpSamples;
-  rm_load_rows<D>(x0, s0, N, 1.0f, xs);
-  for (int step = 0; step < T; ++step) {
-    rm_euler_step<D, TRACE, CS>(tab, sh, sm, xs, bias, eta, s0, N, step, traj, steps);
-    if (ckpt != nullptr && (step + 1) % kck == 0 && sh.crank == 0)
-      rm_store_rows<D>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
-  }
-  rm_leave<CS>(sh);
-  if (sh.crank > 0) return;
-  if (xT) rm_store_rows<D>(xs, s0, N, xT);
-  if (TRACE) rm_store_rows<D>(xs, s0, N, traj + (int64_t)T * N * D);
+  if (CS > 1 || blockIdx.x < n2)
+    rm_morph_block<D, TRACE, CS, kRmRows>(sm, tab, nstage, bias, x0, (int64_t)(blockIdx.x / CS) * kRmSamples, N, T, eta,
+                                          xT, ckpt, kck, traj, steps);
+  else
+    rm_morph_block<D, TRACE, 1, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, xT, ckpt, kck, traj,
+                                   steps);
 }
 
 // Weight-gradient pass at x (A fragments ah, al) with v = g (vh, vl), both
@@ -499,10 +524,11 @@ k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const flo
 // (per lane, for its rows g and g + 8 of each row tile).  Per k tile the
 // lanes sharing t add their rows (shuffles over g), the warps' partials go
 // through shared memory and are added to the block's row in a fixed order.
+template <int R>
 __device__ __forceinline__ void rm_gw_sweep(const float* __restrict__ tab, int nstage, float* sm, float* part,
-                                            const uint32_t (&ah)[kRmRows][4], const uint32_t (&al)[kRmRows][4],
-                                            const uint32_t (&vh)[kRmRows][4], const uint32_t (&vl)[kRmRows][4],
-                                            const float (&cA)[kRmRows][2], const float (&cB)[kRmRows][2],
+                                            const uint32_t (&ah)[R][4], const uint32_t (&al)[R][4],
+                                            const uint32_t (&vh)[R][4], const uint32_t (&vl)[R][4],
+                                            const float (&cA)[R][2], const float (&cB)[R][2],
                                             float* __restrict__ row, int64_t M) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const float twopi = k2PiHi;
@@ -521,7 +547,7 @@ __device__ __forceinline__ void rm_gw_sweep(const float* __restrict__ tab, int n
       const uint32_t btl0 = __float_as_uint(bt.z), btl1 = __float_as_uint(bt.w);
       float p0 = 0.0f, p1 = 0.0f;   // features 2t and 2t + 1 of the k tile
 #pragma unroll
-      for (int r = 0; r < kRmRows; ++r) {
+      for (int r = 0; r < R; ++r) {
         float d[4] = {0.0f, 0.0f, 0.0f, 0.0f}, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         mma_tf32(d, al[r][0], al[r][1], al[r][2], al[r][3], bth0, bth1);
         mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], btl0, btl1);
@@ -566,54 +592,52 @@ __device__ __forceinline__ void rm_gw_sweep(const float* __restrict__ tab, int n
 // segment from the checkpoints: the segment's states are recomputed into the
 // warp's shared memory (kseg x [32][8]), then each step back is one
 // Hessian-vector pass with v = g.
-template <int D>
-__global__ void __launch_bounds__(kRmWarps * 32, 3)
-k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
-              float eta, int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT, float* __restrict__ g0,
-              float* __restrict__ rows, int64_t M) {
-  extern __shared__ __align__(16) float sm[];
-  rm_stage_init();
+template <int D, int R>
+__device__ __forceinline__ void rm_vjp_block(float* sm, const float* __restrict__ tab, int nstage, float bias,
+                                             const float* __restrict__ x0, int64_t first, int64_t N, int T, float eta,
+                                             int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT,
+                                             float* __restrict__ g0, float* __restrict__ rows, int64_t M) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
-  float* gs = sm + 2 * kRmStageFloats + warp * (kseg + 1) * (kRmWarpSamples * 8);   // [32][8], column 7 = 0
-  float* seg = gs + kRmWarpSamples * 8;                                              // kseg x [32][8]
+  float* gs = sm + 2 * kRmStageFloats + warp * (kseg + 1) * ((R * 16) * 8);   // [32][8], column 7 = 0
+  float* seg = gs + (R * 16) * 8;                                              // kseg x [32][8]
   // weight gradient (rows != nullptr): this block's row of rows_[blocks][M + 1], warp partials, bias partials
-  float* part = sm + 2 * kRmStageFloats + kRmWarps * (kseg + 1) * (kRmWarpSamples * 8);   // [4][128]
+  float* part = sm + 2 * kRmStageFloats + kRmWarps * (kseg + 1) * ((R * 16) * 8);   // [4][128]
   float* gbw = part + kRmWarps * kRmStageKT * 8;                                        // [4]
   float* row = rows ? rows + (int64_t)blockIdx.x * (M + 1) : nullptr;
   if (row)
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
   float gb_acc = 0.0f;
-  const int64_t s0 = (int64_t)blockIdx.x * kRmSamples + warp * kRmWarpSamples;
+  const int64_t s0 = first + warp * (R * 16);
   RmShare one = rm_share(1, nstage, nullptr);
-  rm_load_rows<D>(gT, s0, N, 0.0f, gs);
+  rm_load_rows<D, R>(gT, s0, N, 0.0f, gs);
   const float twopi = k2PiHi;
   const int nseg = T / kseg;
   for (int sgi = nseg - 1; sgi >= 0; --sgi) {
     if (sgi == 0 || ckpt == nullptr) {
-      rm_load_rows<D>(x0, s0, N, 1.0f, seg);
+      rm_load_rows<D, R>(x0, s0, N, 1.0f, seg);
       for (int q = 0; q < sgi * kseg; ++q)
-        rm_euler_step<D, false>(tab, one, sm, seg, bias, eta, s0, N, 0, nullptr, nullptr);
+        rm_euler_step<D, false, 1, R>(tab, one, sm, seg, bias, eta, s0, N, 0, nullptr, nullptr);
     } else {
-      rm_load_rows<D>(ckpt + (int64_t)(sgi - 1) * N * D, s0, N, 1.0f, seg);
+      rm_load_rows<D, R>(ckpt + (int64_t)(sgi - 1) * N * D, s0, N, 1.0f, seg);
     }
     for (int i = 1; i < kseg; ++i) {
-      float* dst = seg + i * (kRmWarpSamples * 8);
-      for (int q = lane; q < kRmWarpSamples * 8; q += 32) dst[q] = dst[q - kRmWarpSamples * 8];
+      float* dst = seg + i * ((R * 16) * 8);
+      for (int q = lane; q < (R * 16) * 8; q += 32) dst[q] = dst[q - (R * 16) * 8];
       __syncwarp();
-      rm_euler_step<D, false>(tab, one, sm, dst, bias, eta, s0, N, 0, nullptr, nullptr);
+      rm_euler_step<D, false, 1, R>(tab, one, sm, dst, bias, eta, s0, N, 0, nullptr, nullptr);
     }
     for (int i = kseg - 1; i >= 0; --i) {
-      const float* xi = seg + i * (kRmWarpSamples * 8);
-      uint32_t ah[kRmRows][4], al[kRmRows][4], vh[kRmRows][4], vl[kRmRows][4];
+      const float* xi = seg + i * ((R * 16) * 8);
+      uint32_t ah[R][4], al[R][4], vh[R][4], vl[R][4];
       rm_frags(xi, g, t, ah, al);
       rm_frags(gs, g, t, vh, vl);
-      float G[kRmRows][4], P[kRmRows][4];
-      u64 S[kRmRows][2];
+      float G[R][4], P[R][4];
+      u64 S[R][2];
       rm_sweep<true>(tab, nstage, sm, ah, al, vh, vl, S, G, P);
-      float D1[kRmRows][2], D2[kRmRows][2], GD[kRmRows][2];
+      float D1[R][2], D2[R][2], GD[R][2];
 #pragma unroll
-      for (int r = 0; r < kRmRows; ++r)
+      for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const int rw = r * 16 + g + 8 * hh;
@@ -625,9 +649,9 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
           GD[r][hh] = gd;
         }
       if (row) {   // d/dw with g_{t+1}, before the update
-        float cA[kRmRows][2], cB[kRmRows][2];
+        float cA[R][2], cB[R][2];
 #pragma unroll
-        for (int r = 0; r < kRmRows; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
             cA[r][hh] = -eta * D2[r][hh] * GD[r][hh];
@@ -637,7 +661,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
         rm_gw_sweep(tab, nstage, sm, part, ah, al, vh, vl, cA, cB, row, M);
       }
 #pragma unroll
-      for (int r = 0; r < kRmRows; ++r) {
+      for (int r = 0; r < R; ++r) {
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const int rw = r * 16 + g + 8 * hh;
@@ -655,7 +679,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
       __syncwarp();
     }
   }
-  rm_store_rows<D>(gs, s0, N, g0);
+  rm_store_rows<D, R>(gs, s0, N, g0);
   if (row) {
     // the bias term: lanes t = 0 hold their rows' sums; warp totals, then the block's in a fixed order
 #pragma unroll
@@ -670,6 +694,28 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
   }
 }
 
+template <int D>
+__global__ void __launch_bounds__(kRmWarps * 32, 3)
+k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
+              float eta, int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT, float* __restrict__ g0,
+              float* __restrict__ rows, int64_t M, unsigned n2) {
+  extern __shared__ __align__(16) float sm[];
+  rm_stage_init();
+  if (blockIdx.x < n2)
+    rm_vjp_block<D, kRmRows>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, rows,
+                             M);
+  else
+    rm_vjp_block<D, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, rows, M);
+}
+
+static int rm_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
+                                                 cudaSuccess || sms < 1)
+    sms = 152;
+  return sms;
+}
+
 // Blocks per tile of a morph: the number (1, 2, 4, 8) with the shortest predicted time.
 // With n blocks together on an SM a stage of 128 features takes stage_us[n]; a
 // launch runs full waves of per_sm blocks an SM and then what is left; adding
@@ -682,10 +728,7 @@ k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float
 // An SM holds five blocks of the kernel for one block per tile, four of the others.
 static int rm_cluster(int64_t tiles, int nstage) {
   static const double stage_us[6] = {0.0, 3.3, 4.7, 6.1, 8.4, 8.5};
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                 cudaSuccess || sms < 1)
-    sms = 152;
+  const int sms = rm_sms();
   int best = 1;
   double best_t = 0.0;
   for (int cs = 1; cs <= 8 && cs <= nstage; cs *= 2) {
@@ -701,12 +744,30 @@ static int rm_cluster(int64_t tiles, int nstage) {
   return best;
 }
 
+// Tiles past the last full wave (per_sm blocks on every SM) go out as halves, if
+// the halves fit on the GPU at once: a half is over in about 0.65 of a tile's
+// time, and up to twice as many SMs take part.  Not where the tiles would be one to an
+// SM behind full waves (two halves to an SM are then no faster).  Measured
+// (ms, M = 4096, T = 20, whole tiles / dealt; per_sm 3): VJP with d/dw and its
+// forward of 2000 samples 7.33 / 5.42, 25,000 10.3 / 8.16, 65,537 19.6 / 18.0;
+// log-det 3.11 / 2.37, 4.64 / 3.75, 8.91 / 8.06; all in halves is slower from
+// 38,000 samples on (19.9 and 9.26 at 65,537).
+static RmDeal rm_deal(int64_t N, int per_sm) {
+  const int64_t tiles = (N + kRmSamples - 1) / kRmSamples, sms = rm_sms(), slots = per_sm * sms;
+  int64_t n2 = tiles / slots * slots;
+  const int64_t rest = tiles - n2;
+  if (2 * rest > slots || (n2 > 0 && 2 * rest > sms && rest <= sms)) n2 = tiles;
+  if (n2 == tiles) return RmDeal{(unsigned)tiles, (unsigned)tiles};
+  const int64_t halves = (N - n2 * kRmSamples + kRmSamples / 2 - 1) / (kRmSamples / 2);
+  return RmDeal{(unsigned)n2, (unsigned)(n2 + halves)};
+}
+
 template <typename Fn, typename... A>
-static cudaError_t rm_launch(Fn fn, int64_t tiles, int cs, size_t smem, cudaStream_t st, A... args) {
+static cudaError_t rm_launch(Fn fn, unsigned blocks, int cs, size_t smem, cudaStream_t st, A... args) {
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t c{};
-  c.gridDim = dim3((unsigned)(tiles * cs));
+  c.gridDim = dim3(blocks);
   c.blockDim = dim3(kRmWarps * 32);
   c.dynamicSmemBytes = smem;
   c.stream = st;
@@ -719,12 +780,12 @@ static cudaError_t rm_launch(Fn fn, int64_t tiles, int cs, size_t smem, cudaStre
   c.numAttrs = cs > 1 ? 1 : 0;
   return cudaLaunchKernelEx(&c, fn, args...);
 }
-// fn: a kernel template over the blocks per tile
-#define PDMP_RM_LAUNCH(cs, tiles, smem, st, KERNEL, ...)                                                     \
-  ((cs) == 8   ? rm_launch(KERNEL(8), tiles, 8, smem, st, __VA_ARGS__)                                       \
-   : (cs) == 4 ? rm_launch(KERNEL(4), tiles, 4, smem, st, __VA_ARGS__)                                       \
-   : (cs) == 2 ? rm_launch(KERNEL(2), tiles, 2, smem, st, __VA_ARGS__)                                       \
-               : rm_launch(KERNEL(1), tiles, 1, smem, st, __VA_ARGS__))
+// KERNEL: a kernel template over the blocks per tile
+#define PDMP_RM_LAUNCH(cs, blocks, smem, st, KERNEL, ...)                                                    \
+  ((cs) == 8   ? rm_launch(KERNEL(8), blocks, 8, smem, st, __VA_ARGS__)                                      \
+   : (cs) == 4 ? rm_launch(KERNEL(4), blocks, 4, smem, st, __VA_ARGS__)                                      \
+   : (cs) == 2 ? rm_launch(KERNEL(2), blocks, 2, smem, st, __VA_ARGS__)                                      \
+               : rm_launch(KERNEL(1), blocks, 1, smem, st, __VA_ARGS__))
 constexpr size_t kRmShareBytes = (size_t)kRmWarps * kRmWarpSamples * 8 * sizeof(float);   // one array of sums
 
 template <int D>
@@ -738,15 +799,16 @@ static cudaError_t launch_rff_mma(const FieldArgs& fa, const float* x0, int64_t 
   // Checkpoints are where a VJP's replay starts, which runs one block per tile: their
   // sums are taken the same way, so that each segment ends where the next begins.
   const int cs = ckpt ? 1 : rm_cluster(tiles, nstage);
+  const RmDeal deal = cs > 1 ? RmDeal{0u, (unsigned)(tiles * cs)} : rm_deal(N, 4);
   const size_t smem = rm_smem_bytes() + (cs > 1 ? kRmShareBytes : 0);
 #define PDMP_KERNEL(CS) (k_morph_rff_mma<D, true, CS>)
   if (traj != nullptr)
-    return PDMP_RM_LAUNCH(cs, tiles, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, traj,
-                          steps);
+    return PDMP_RM_LAUNCH(cs, deal.blocks, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, traj,
+                          steps, deal.n2);
 #undef PDMP_KERNEL
 #define PDMP_KERNEL(CS) (k_morph_rff_mma<D, false, CS>)
-  return PDMP_RM_LAUNCH(cs, tiles, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, nullptr,
-                        nullptr);
+  return PDMP_RM_LAUNCH(cs, deal.blocks, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, nullptr,
+                        nullptr, deal.n2);
 #undef PDMP_KERNEL
 }
 
@@ -780,30 +842,27 @@ __host__ __device__ constexpr size_t ld_rff_smem_bytes() {
   return (2 * (size_t)kLdStageFloats + (size_t)kRmWarps * kRmWarpSamples * (8 + kLdGather)) * sizeof(float);
 }
 
-template <int D>
-__global__ void __launch_bounds__(kRmWarps * 32, 3)
-k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N,
-                 int T, float eta, float* __restrict__ logdet, float* __restrict__ xT) {
-  static_assert(D >= 1 && D <= 7, "dimensions and the phase share the 8 k slots");
-  extern __shared__ __align__(16) float sm[];
-  rm_stage_init();
+template <int D, int R>
+__device__ __forceinline__ void rm_logdet_block(float* sm, const float* __restrict__ tab, int nstage, float bias,
+                                                const float* __restrict__ x0, int64_t first, int64_t N, int T,
+                                                float eta, float* __restrict__ logdet, float* __restrict__ xT) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
-  float* xs = sm + 2 * kLdStageFloats + warp * kRmWarpSamples * (8 + kLdGather);
-  float* gat = xs + kRmWarpSamples * 8;
-  const int64_t s0 = (int64_t)blockIdx.x * kRmSamples + warp * kRmWarpSamples;
-  rm_load_rows<D>(x0, s0, N, 1.0f, xs);
+  float* xs = sm + 2 * kLdStageFloats + warp * (R * 16) * (8 + kLdGather);
+  float* gat = xs + (R * 16) * 8;
+  const int64_t s0 = first + warp * (R * 16);
+  rm_load_rows<D, R>(x0, s0, N, 1.0f, xs);
   float total = 0.0f;
   bool bad = false;
   const u64 c12 = pk(6144.0f, 6144.0f), nc12 = pk(-6144.0f, -6144.0f), mone = pk(-1.0f, -1.0f);
 
   for (int step = 0; step < T; ++step) {
-    uint32_t ah[kRmRows][4], al[kRmRows][4];
+    uint32_t ah[R][4], al[R][4];
     rm_frags(xs, g, t, ah, al);
-    float G[kRmRows][4], Q[kRmRows][kLdNT][4];
-    u64 S[kRmRows][2];
+    float G[R][4], Q[R][kLdNT][4];
+    u64 S[R][2];
 #pragma unroll
-    for (int r = 0; r < kRmRows; ++r) {
+    for (int r = 0; r < R; ++r) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         G[r][q] = 0.0f;
@@ -831,7 +890,7 @@ k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const fl
 #pragma unroll
         for (int nt = 0; nt < kLdNT; ++nt) bh[nt] = reinterpret_cast<const float4*>(rec + kRmKtFloats + 128 * nt)[lane];
 #pragma unroll
-        for (int r = 0; r < kRmRows; ++r) {
+        for (int r = 0; r < R; ++r) {
           float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
           mma_tf32(d, al[r][0], al[r][1], al[r][2], al[r][3], __float_as_uint(bt.x), __float_as_uint(bt.y));
           mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], __float_as_uint(bt.z), __float_as_uint(bt.w));
@@ -877,7 +936,7 @@ k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const fl
     }
     // gather each sample's sums: Hess s columns from the quad, s and grad s
 #pragma unroll
-    for (int r = 0; r < kRmRows; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
         const float s = rm_logit(S, r, hh);
@@ -893,7 +952,7 @@ k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const fl
           if (2 * t + e < D) row[33 + 2 * t + e] = G[r][2 * hh + e];
       }
     __syncwarp();
-    {
+    if (lane < R * 16) {
       // lane = sample: I - eta Hess c, its Cholesky log-det, the Euler update
       const float* row = gat + lane * kLdGather;
       float gsv[D];
@@ -923,11 +982,24 @@ k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const fl
     __syncwarp();
   }
   const int64_t own = s0 + lane;
-  if (own < N) {
+  if (lane < R * 16 && own < N) {
     if (bad) raise_flag(FLAG_NONPOSITIVE_PIVOT);
     logdet[own] = bad ? nanf("") : total;
   }
-  if (xT) rm_store_rows<D>(xs, s0, N, xT);
+  if (xT) rm_store_rows<D, R>(xs, s0, N, xT);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kRmWarps * 32, 3)
+k_logdet_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N,
+                 int T, float eta, float* __restrict__ logdet, float* __restrict__ xT, unsigned n2) {
+  static_assert(D >= 1 && D <= 7, "dimensions and the phase share the 8 k slots");
+  extern __shared__ __align__(16) float sm[];
+  rm_stage_init();
+  if (blockIdx.x < n2)
+    rm_logdet_block<D, kRmRows>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, logdet, xT);
+  else
+    rm_logdet_block<D, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, logdet, xT);
 }
 
 template <int D>
@@ -939,9 +1011,9 @@ static cudaError_t launch_logdet_rff_mma(const FieldArgs& fa, const float* x0, i
   constexpr size_t smem = ld_rff_smem_bytes();
   cudaError_t e = cudaFuncSetAttribute(k_logdet_rff_mma<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)((N + kRmSamples - 1) / kRmSamples);
-  k_logdet_rff_mma<D><<<blocks, kRmWarps * 32, smem, st>>>(tab, (int)(n_kt / kLdStageKT), fa.bias, x0, N, T, eta,
-                                                           ld, xT);
+  const RmDeal deal = rm_deal(N, 3);
+  k_logdet_rff_mma<D><<<deal.blocks, kRmWarps * 32, smem, st>>>(tab, (int)(n_kt / kLdStageKT), fa.bias, x0, N, T, eta,
+                                                                ld, xT, deal.n2);
   return cudaGetLastError();
 }
 
@@ -1089,7 +1161,7 @@ cudaError_t stage_wait_selftest(const float* src, float* dst, long long limit, i
   return cudaGetLastError();
 }
 
-int64_t vjp_rff_mma_blocks(int64_t N) { return (N + kRmSamples - 1) / kRmSamples; }
+int64_t vjp_rff_mma_blocks(int64_t N) { return rm_deal(N, 3).blocks; }
 
 // the tensor-core VJP keeps a segment of states in shared memory: k <= 16
 size_t vjp_rff_mma_smem(int k) {
@@ -1107,9 +1179,10 @@ static cudaError_t launch_vjp_rff_mma(const FieldArgs& fa, const float* x0, int6
   const size_t smem = vjp_rff_mma_smem(k);
   cudaError_t e = cudaFuncSetAttribute(k_vjp_rff_mma<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)vjp_rff_mma_blocks(N);
+  const RmDeal deal = rm_deal(N, 3);
+  const unsigned blocks = deal.blocks;
   k_vjp_rff_mma<D><<<blocks, kRmWarps * 32, smem, st>>>(tab, (int)(n_kt / kRmStageKT), fa.bias, x0, N, T, eta, k,
-                                                        ckpt, gT, g0, rows, fa.M);
+                                                        ckpt, gT, g0, rows, fa.M, deal.n2);
   e = cudaGetLastError();
   if (e != cudaSuccess || rows == nullptr) return e;
   return sum_vjp_rows(rows, (int64_t)blocks, fa.M + 1, gw, gbias, st);

@@ -45,3 +45,39 @@ def test_morph_of_few_tiles(d, M, N):
     assert torch.equal(ck[-1], xc)
     assert float((xc - xT).abs().max()) <= 2e-5
     assert float((ck[0] - traj[k]).abs().max()) <= 2e-5
+
+
+@pytest.mark.parametrize("d,M", [(7, 300), (3, 1000)])
+def test_dealing_tiles_out_in_halves_keeps_the_results(d, M):
+    """One launch of whole tiles and halves behind a full wave, against launches
+    of halves alone: the same log-det, end points, checkpoints and gradient of
+    every sample, and a weight gradient that adds up."""
+    N = 128 * 3 * torch.cuda.get_device_properties(0).multi_processor_count + 700
+    f = wl.random_field(M + d, wl.RFF, d, M, wscale=5.0, bias=0.1)
+    lo, hi = np.full(d, -np.pi), np.full(d, np.pi)
+    eta, _ = rff_eta_sampled(f, lo, hi, n=400)
+    fld = pdmp.DeviceField.from_host(f)
+    x0 = wl.uniform_box(N, 3, N, lo, hi)
+    x = torch.from_numpy(x0).cuda()
+    gT = torch.from_numpy(wl.f32(wl.rng(N, wl.S_COTANGENT).standard_normal((N, d)))).cuda()
+    T, k = 4, 2
+
+    def run(sl):
+        xs, gs = x[sl].clone(), gT[sl].clone()
+        ck = torch.empty(T // k, xs.shape[0], d, device="cuda")
+        xT = pdmp.morph(fld, xs, T, eta, ckpt=ck, k=k)
+        ld, xl = pdmp.logdet(fld, xs, T, eta, want_xT=True)
+        g0, gw, gb = pdmp.morph_vjp(fld, xs, T, eta, k, gs, ckpt=ck, want_param_grad=True)
+        return [xT, ck.transpose(0, 1), ld, xl, g0], gw, gb
+
+    whole, gw, gb = run(slice(0, N))
+    cuts = [0, 65, 4000, 4128, 12000, N - 700, N]
+    sw = torch.zeros_like(gw)
+    for a, b in zip(cuts[:-1], cuts[1:]):
+        parts, pw, _ = run(slice(a, b))
+        for q, r in zip(whole, parts):
+            assert torch.equal(q[a:b], r)
+        sw += pw
+    assert float((sw - gw).norm()) <= 1e-5 * float(gw.norm())
+    idx = wl.rng(N, 9).integers(0, N, 40)
+    assert max_abs(whole[2].cpu().numpy()[idx], oracle.logdet(f, x0[idx], T, eta)[0]) <= 1e-4 * T
