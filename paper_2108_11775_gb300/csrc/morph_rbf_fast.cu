@@ -40,8 +40,12 @@ k_morph_rbf_fast(TileArgs a) {
 // Samples per lane.  A launch of fewer 320-sample tiles than fit on the GPU at
 // once (3 per SM) leaves SMs idle; it takes 128-sample tiles instead (16
 // warps per SM).  Measured on a 3-D field (M = 8192, T = 40): 2^16 samples
-// 9.3 ms against 13.2 ms; from one wave of 320-sample tiles up (197,641 and
-// 2^18 samples) the larger tiles are as fast or faster.
+// 9.3 ms against 13.2 ms; from one wave of 320-sample tiles up the larger tiles
+// are as fast or faster in 2-D.  In 3-D a tile's box shrinks slower with the number
+// of samples, and small boxes have fewer near groups, so small tiles are kept for
+// two thirds more samples (200,000 samples in boxes of 5^3 / 10^3, gamma = 8, M =
+// 4096, T = 10: 2.11 / 1.46 ms against 2.21 / 2.04; 400,000: 3.60 / 2.04 against
+// 3.52 / 2.86; 2^20: 8.28 / 4.46 against 7.40 / 4.12).
 constexpr int kSmallK = 4;
 
 static int num_sms() {
@@ -90,7 +94,7 @@ template <int D, bool TRACE>
 static cudaError_t launch_tiles(const TileArgs& a, int64_t N, cudaStream_t st) {
   const int64_t sms = num_sms();
   const int64_t tiles = (N + FastShape::kTile - 1) / FastShape::kTile;
-  if (tiles >= FastShape::kMinBlocks * sms) return launch_shape<D, TRACE, FastShape::kK, 1>(a, N, st);
+  if (tiles >= (D == 3 ? 5 : FastShape::kMinBlocks) * sms) return launch_shape<D, TRACE, FastShape::kK, 1>(a, N, st);
   const int64_t small = (N + Shape<4, kSmallK>::kTile - 1) / Shape<4, kSmallK>::kTile;
   if (small <= sms) return launch_shape<D, TRACE, kSmallK, 4>(a, N, st);
   if (small <= 2 * sms) return launch_shape<D, TRACE, kSmallK, 2>(a, N, st);
