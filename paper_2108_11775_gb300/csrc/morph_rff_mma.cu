@@ -30,11 +30,16 @@
 namespace pdmp {
 
 // Measured on the 7-D workload (N = 2^20, M = 4096, T = 20): two row tiles
-// a warp, k tiles unrolled by two and stages of 16 k tiles ran fastest among
-// 1 / 2 / 4 row tiles, unroll 1 / 2 / 4 and 16 / 32 k tiles a stage.
+// a warp and stages of 16 k tiles ran fastest among 1 / 2 / 4 row tiles and 16 /
+// 32 k tiles a stage.  A k tile is a chain of three MMAs, sines and cosines and
+// three MMAs more, and three or four warps a scheduler do not cover it: with k
+// tiles unrolled by 1 / 2 / 4 / 8 the VJP with d/dw of 65,537 samples takes 18.2 /
+// 16.6 / 16.0 / 16.2 ms (of 2000, one row tile a warp, 5.8 / 4.5 / 4.0 / 3.8), the
+// morph of 131,072 6.69 / 6.28 / 6.17 / 6.28.  The log-det's k tiles by 1 / 2 / 4:
+// 14.9 / 14.2 / 14.4 ms for 131,072 samples, 2.31 / 1.85 / 1.65 for 2000.
 constexpr int kRmWarps = 4;
 constexpr int kRmRows = 2;                              // 16-sample row tiles per warp
-constexpr int kRmUnroll = 2;
+constexpr int kRmUnroll = 4;   // twice that with one row tile a warp
 constexpr int kRmWarpSamples = kRmRows * 16;
 constexpr int kRmSamples = kRmWarps * kRmWarpSamples;   // per block
 constexpr int kRmStageKT = 16;                          // k tiles (8 features each) per stage
@@ -288,7 +293,7 @@ __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nsta
     if (st + 1 < nstage)
       rm_stage_load(tab + (size_t)(st + 1) * kRmStageFloats, sm + ((st + 1) & 1) * kRmStageFloats);
     const float* sb = sm + (st & 1) * kRmStageFloats;
-#pragma unroll kRmUnroll
+#pragma unroll (R == 1 ? 2 * kRmUnroll : kRmUnroll)
     for (int kt = 0; kt < kRmStageKT; ++kt) {
       const float* rec = sb + kt * kRmKtFloats;
       const float4 bt = reinterpret_cast<const float4*>(rec)[lane];
@@ -521,9 +526,11 @@ k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const flo
 // block's sum over its samples of
 //   cA_n cos(theta_nm) + cB_n (grad phi_m . g_n),   grad phi_m . g = -sin(theta_m) omega_m . g,
 // with cA_n = -eta sigma''(s_n) (grad s_n . g_n) and cB_n = -eta sigma'(s_n)
-// (per lane, for its rows g and g + 8 of each row tile).  Per k tile the
-// lanes sharing t add their rows (shuffles over g), the warps' partials go
-// through shared memory and are added to the block's row in a fixed order.
+// (per lane, for its rows g and g + 8 of each row tile).  The lanes sharing t
+// add their rows, four k tiles at a time: each step of the exchange hands over
+// half of the eight sums, 7 shuffles instead of 24 and four chains in flight
+// (VJP of 65,537 samples 18.0 -> 16.6 ms).  The warps' partials go through shared
+// memory and are added to the block's row in a fixed order.
 template <int R>
 __device__ __forceinline__ void rm_gw_sweep(const float* __restrict__ tab, int nstage, float* sm, float* part,
                                             const uint32_t (&ah)[R][4], const uint32_t (&al)[R][4],
@@ -541,39 +548,51 @@ __device__ __forceinline__ void rm_gw_sweep(const float* __restrict__ tab, int n
       rm_stage_load(tab + (size_t)(st + 1) * kRmStageFloats, sm + ((st + 1) & 1) * kRmStageFloats);
     const float* sb = sm + (st & 1) * kRmStageFloats;
 #pragma unroll 1
-    for (int kt = 0; kt < kRmStageKT; ++kt) {
-      const float4 bt = reinterpret_cast<const float4*>(sb + kt * kRmKtFloats)[lane];
-      const uint32_t bth0 = __float_as_uint(bt.x), bth1 = __float_as_uint(bt.y);
-      const uint32_t btl0 = __float_as_uint(bt.z), btl1 = __float_as_uint(bt.w);
-      float p0 = 0.0f, p1 = 0.0f;   // features 2t and 2t + 1 of the k tile
+    for (int k0 = 0; k0 < kRmStageKT; k0 += 4) {
+      float v[8];   // feature 2t + (e & 1) of k tile k0 + (e >> 1)
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        float d[4] = {0.0f, 0.0f, 0.0f, 0.0f}, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        mma_tf32(d, al[r][0], al[r][1], al[r][2], al[r][3], bth0, bth1);
-        mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], btl0, btl1);
-        mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], bth0, bth1);
-        mma_tf32(o, vl[r][0], vl[r][1], vl[r][2], vl[r][3], bth0, bth1);
-        mma_tf32(o, vh[r][0], vh[r][1], vh[r][2], vh[r][3], btl0, btl1);
-        mma_tf32(o, vh[r][0], vh[r][1], vh[r][2], vh[r][3], bth0, bth1);
-        float f[4];
-        upk(rm_turns_to_rad(pk(d[0], d[1])), f[0], f[1]);
-        upk(rm_turns_to_rad(pk(d[2], d[3])), f[2], f[3]);
-        // element q: row g + 8 (q >> 1), feature 2t + (q & 1)
+      for (int e = 0; e < 4; ++e) {
+        const int kt = k0 + e;
+        const float4 bt = reinterpret_cast<const float4*>(sb + kt * kRmKtFloats)[lane];
+        const uint32_t bth0 = __float_as_uint(bt.x), bth1 = __float_as_uint(bt.y);
+        const uint32_t btl0 = __float_as_uint(bt.z), btl1 = __float_as_uint(bt.w);
+        float p0 = 0.0f, p1 = 0.0f;   // features 2t and 2t + 1 of the k tile
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float c = fmaf(-cB[r][q >> 1] * twopi * sin_approx(f[q]), o[q], cA[r][q >> 1] * cos_approx(f[q]));
-          if (q & 1) p1 += c; else p0 += c;
+        for (int r = 0; r < R; ++r) {
+          float d[4] = {0.0f, 0.0f, 0.0f, 0.0f}, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          mma_tf32(d, al[r][0], al[r][1], al[r][2], al[r][3], bth0, bth1);
+          mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], btl0, btl1);
+          mma_tf32(d, ah[r][0], ah[r][1], ah[r][2], ah[r][3], bth0, bth1);
+          mma_tf32(o, vl[r][0], vl[r][1], vl[r][2], vl[r][3], bth0, bth1);
+          mma_tf32(o, vh[r][0], vh[r][1], vh[r][2], vh[r][3], btl0, btl1);
+          mma_tf32(o, vh[r][0], vh[r][1], vh[r][2], vh[r][3], bth0, bth1);
+          float f[4];
+          upk(rm_turns_to_rad(pk(d[0], d[1])), f[0], f[1]);
+          upk(rm_turns_to_rad(pk(d[2], d[3])), f[2], f[3]);
+          // element q: row g + 8 (q >> 1), feature 2t + (q & 1)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float c = fmaf(-cB[r][q >> 1] * twopi * sin_approx(f[q]), o[q], cA[r][q >> 1] * cos_approx(f[q]));
+            if (q & 1) p1 += c; else p0 += c;
+          }
+        }
+        v[2 * e] = p0;
+        v[2 * e + 1] = p1;
+      }
+      // the lanes sharing t add up; each step hands half of the values over
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1) {
+        const int off = 16 / h;   // 4, 8, 16
+        const bool upper = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+          const float keep = upper ? v[h + i] : v[i], give = upper ? v[i] : v[h + i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
         }
       }
-#pragma unroll
-      for (int off = 4; off < 32; off <<= 1) {
-        p0 += __shfl_xor_sync(0xffffffffu, p0, off);
-        p1 += __shfl_xor_sync(0xffffffffu, p1, off);
-      }
-      if (g == 0) {
-        part[warp * (kRmStageKT * 8) + kt * 8 + 2 * t] = p0;
-        part[warp * (kRmStageKT * 8) + kt * 8 + 2 * t + 1] = p1;
-      }
+      // lane g holds value e = 4 (g & 1) + 2 (g >> 1 & 1) + (g >> 2)
+      const int e = 4 * (g & 1) + 2 * (g >> 1 & 1) + (g >> 2);
+      part[warp * (kRmStageKT * 8) + (k0 + (e >> 1)) * 8 + 2 * t + (e & 1)] = v[0];
     }
     __syncthreads();   // every warp's partials of this stage
     for (int fi = threadIdx.x; fi < kRmStageKT * 8; fi += kRmWarps * 32) {
@@ -880,7 +899,7 @@ __device__ __forceinline__ void rm_logdet_block(float* sm, const float* __restri
         rm_stage_load<kLdStageFloats>(tab + (size_t)(st + 1) * kLdStageFloats,
                                       sm + ((st + 1) & 1) * kLdStageFloats);
       const float* sb = sm + (st & 1) * kLdStageFloats;
-#pragma unroll 1
+#pragma unroll (R == 1 ? 4 : 2)
       for (int kt = 0; kt < kLdStageKT; ++kt) {
         const float* rec = sb + kt * kLdKtFloats;
         const float4 bt = reinterpret_cast<const float4*>(rec)[lane];
