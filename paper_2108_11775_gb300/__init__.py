@@ -642,12 +642,20 @@ def occupancy_query(field: DeviceField, x: torch.Tensor, want=("c", "s", "grad")
     c = torch.empty(N, device=x.device, dtype=torch.float32) if "c" in want else None
     s = torch.empty(N, device=x.device, dtype=torch.float32) if "s" in want else None
     g = torch.empty(N, d, device=x.device, dtype=torch.float32) if "grad" in want else None
-    f = field.struct()
-    # long sweeps of 2-D / 3-D RBF fields run on sorted tiles, which want a workspace
-    nbytes = int(lib().pdmp_occupancy_query_workspace(ctypes.byref(f), N))
-    ws = torch.empty(nbytes, dtype=torch.uint8, device=x.device) if nbytes else None
-    st = lib().pdmp_occupancy_query_ws(ctypes.byref(f), _ptr(x, shape=(N, d), name="x"), N, _ptr(c), _ptr(s), _ptr(g),
-                                       ctypes.c_void_p(ws.data_ptr()) if nbytes else None, nbytes, _stream())
+    f, L = field.struct(), lib()
+    # Long sweeps of 2-D / 3-D RBF fields run on sorted tiles, which want a
+    # workspace; the library says how much, and is not asked about calls too
+    # small for it (a few microseconds of a call of thirty).
+    nbytes = 0
+    if field.kind == RBF and (field.M >= 1024 or N * field.M >= 1 << 27):
+        nbytes = int(L.pdmp_occupancy_query_workspace(ctypes.byref(f), N))
+    xp = _ptr(x, shape=(N, d), name="x")
+    if nbytes:
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=x.device)
+        st = L.pdmp_occupancy_query_ws(ctypes.byref(f), xp, N, _ptr(c), _ptr(s), _ptr(g),
+                                       ctypes.c_void_p(ws.data_ptr()), nbytes, _stream())
+    else:
+        st = L.pdmp_occupancy_query(ctypes.byref(f), xp, N, _ptr(c), _ptr(s), _ptr(g), _stream())
     _check(st, "pdmp_occupancy_query")
     return {"c": c, "s": s, "grad": g}
 
