@@ -518,8 +518,7 @@ static bool vjp_tiles_eligible(const pdmp_field* f, int64_t N, int32_t k) {
 
 // the per-block rows of the parameter gradient (any VJP kernel's blocks), rounded to 256 bytes
 static size_t vjp_rows_bytes(const pdmp_field* f, int64_t N) {
-  int64_t blocks = pdmp::vjp_blocks(N);
-  if (f->kind == PDMP_KIND_RFF && f->d <= 7) blocks = std::max(blocks, pdmp::vjp_rff_mma_blocks(N));
+  int64_t blocks = std::max(pdmp::vjp_blocks(N), pdmp::vjp_rff_mma_blocks(N));
   if (f->kind == PDMP_KIND_RBF && (f->d == 2 || f->d == 3)) blocks = std::max(blocks, pdmp::vjp_rbf_fast_blocks(f->d, N));
   return (sizeof(float) * (size_t)blocks * (size_t)(f->M + 1) + 255) & ~size_t(255);
 }

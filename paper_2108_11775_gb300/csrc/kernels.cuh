@@ -80,7 +80,8 @@ int64_t vjp_blocks(int64_t N);
 // gw[perm[m]] = sum_b rows[b][m] (m < width - 1), *gbias = sum_b rows[b][width - 1], in block order
 // (perm NULL: the identity)
 cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st,
-                         const int32_t* perm = nullptr);
+                         const int32_t* perm = nullptr,
+                         const float* more = nullptr, int64_t nmore = 0);
 // the tensor-core VJP for RFF fields (d <= 7, segments k <= kVjpMmaMaxSegment; ws: morph_rff_mma_workspace).
 // rows: nullptr, or vjp_rff_mma_blocks(N) x (M + 1) floats for the weight and bias gradient (gw, gbias)
 constexpr int kVjpMmaMaxSegment = 16;

@@ -35,11 +35,15 @@ namespace pdmp {
 // three MMAs more, and three or four warps a scheduler do not cover it: with k
 // tiles unrolled by 1 / 2 / 4 / 8 the VJP with d/dw of 65,537 samples takes 18.2 /
 // 16.6 / 16.0 / 16.2 ms (of 2000, one row tile a warp, 5.8 / 4.5 / 4.0 / 3.8), the
-// morph of 131,072 6.69 / 6.28 / 6.17 / 6.28.  The log-det's k tiles by 1 / 2 / 4:
+// morph of 131,072 6.69 / 6.28 / 6.17 / 6.28.  The morph of many tiles is kept in a
+// kernel of its own, unrolled by two (92 registers, five blocks an SM): 2^20
+// samples 44.8 ms, 46.0 unrolled by four or with the halves' code beside it.  The log-det's k tiles by 1 / 2 / 4:
 // 14.9 / 14.2 / 14.4 ms for 131,072 samples, 2.31 / 1.85 / 1.65 for 2000.
 constexpr int kRmWarps = 4;
 constexpr int kRmRows = 2;                              // 16-sample row tiles per warp
-constexpr int kRmUnroll = 4;   // twice that with one row tile a warp
+template <int R>
+constexpr int kRmUnroll = R == 1 ? 8 : 4;
+constexpr int kRmMorphUnroll = 2;   // the morph's kernel for whole tiles
 constexpr int kRmWarpSamples = kRmRows * 16;
 constexpr int kRmSamples = kRmWarps * kRmWarpSamples;   // per block
 constexpr int kRmStageKT = 16;                          // k tiles (8 features each) per stage
@@ -273,7 +277,7 @@ __device__ __forceinline__ void rm_leave(RmShare& sh) {   // no block leaves whi
 // sum_m cos(theta_m) (omega_m . v / 2 pi) (-w_m omega_m) = (Hess s) v / 2 pi).
 // Block-wide: every warp of the block makes the same sequence of passes.  tab
 // and nstage: the stages of this block (all of them without a cluster).
-template <bool HVP, int R>
+template <bool HVP, int U, int R>
 __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nstage, float* sm,
                                          const uint32_t (&ah)[R][4], const uint32_t (&al)[R][4],
                                          const uint32_t (&vh)[R][4], const uint32_t (&vl)[R][4],
@@ -293,7 +297,7 @@ __device__ __forceinline__ void rm_sweep(const float* __restrict__ tab, int nsta
     if (st + 1 < nstage)
       rm_stage_load(tab + (size_t)(st + 1) * kRmStageFloats, sm + ((st + 1) & 1) * kRmStageFloats);
     const float* sb = sm + (st & 1) * kRmStageFloats;
-#pragma unroll (R == 1 ? 2 * kRmUnroll : kRmUnroll)
+#pragma unroll U
     for (int kt = 0; kt < kRmStageKT; ++kt) {
       const float* rec = sb + kt * kRmKtFloats;
       const float4 bt = reinterpret_cast<const float4*>(rec)[lane];
@@ -413,7 +417,7 @@ __device__ __forceinline__ void rm_combine(RmShare& sh, const u64 (&S)[R][2], fl
 }
 
 // One Euler step of the warp's 16 R samples held in xs ([16 R][8], column 7 = 1).
-template <int D, bool TRACE, int CS, int R>
+template <int D, bool TRACE, int CS, int R, int U = kRmUnroll<R>>
 __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, RmShare& sh, float* sm, float* xs,
                                               float bias, float eta, int64_t s0, int64_t N, int step,
                                               float* __restrict__ traj, float* __restrict__ steps) {
@@ -422,7 +426,7 @@ __device__ __forceinline__ void rm_euler_step(const float* __restrict__ tab, RmS
   rm_frags(xs, g, t, ah, al);
   float G[R][4], P[R][4];
   u64 S[R][2];
-  rm_sweep<false>(CS == 1 ? tab : tab + (size_t)sh.st0 * kRmStageFloats, CS == 1 ? sh.st1 : sh.st1 - sh.st0, sm, ah,
+  rm_sweep<false, U>(CS == 1 ? tab : tab + (size_t)sh.st0 * kRmStageFloats, CS == 1 ? sh.st1 : sh.st1 - sh.st0, sm, ah,
                   al, ah, al, S, G, P);
   float s[R][2];
   if constexpr (CS > 1) rm_combine<CS>(sh, S, s, G);
@@ -484,41 +488,48 @@ __device__ __forceinline__ int64_t rm_first(unsigned b, unsigned n2) {
   return b < n2 ? (int64_t)b * kRmSamples : (int64_t)n2 * kRmSamples + (int64_t)(b - n2) * (kRmSamples / 2);
 }
 
-template <int D, bool TRACE, int CS, int R>
-__device__ __forceinline__ void rm_morph_block(float* sm, const float* __restrict__ tab, int nstage, float bias,
-                                               const float* __restrict__ x0, int64_t first, int64_t N, int T, float eta,
-                                               float* __restrict__ xT, float* __restrict__ ckpt, int kck,
-                                               float* __restrict__ traj, float* __restrict__ steps) {
-  const int warp = threadIdx.x >> 5;
-  float* xs = sm + 2 * kRmStageFloats + warp * (R * 16 * 8);   // [16 R samples][8]: x, 0 .., 1
-  RmShare sh = rm_share(CS, nstage, sm + 2 * kRmStageFloats + kRmWarps * (R * 16 * 8));
-  const int64_t s0 = first + warp * (R * 16);
-  rm_load_rows<D, R>(x0, s0, N, 1.0f, xs);
-  for (int step = 0; step < T; ++step) {
-    rm_euler_step<D, TRACE, CS, R>(tab, sh, sm, xs, bias, eta, s0, N, step, traj, steps);
-    if (ckpt != nullptr && (step + 1) % kck == 0 && sh.crank == 0)
-      rm_store_rows<D, R>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
-  }
-  rm_leave<CS>(sh);
-  if (sh.crank > 0) return;
-  if (xT) rm_store_rows<D, R>(xs, s0, N, xT);
-  if (TRACE) rm_store_rows<D, R>(xs, s0, N, traj + (int64_t)T * N * D);
-}
-
 template <int D, bool TRACE, int CS>
 __global__ void __launch_bounds__(kRmWarps * 32, 4)
 k_morph_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
                 float eta, float* __restrict__ xT, float* __restrict__ ckpt, int kck, float* __restrict__ traj,
-                float* __restrict__ steps, unsigned n2) {
+                float* __restrict__ steps) {
   static_assert(D >= 1 && D <= 7, "dimensions and the phase share the 8 k slots");
   extern __shared__ __align__(16) float sm[];
   rm_stage_init();
-  if (CS > 1 || blockIdx.x < n2)
-    rm_morph_block<D, TRACE, CS, kRmRows>(sm, tab, nstage, bias, x0, (int64_t)(blockIdx.x / CS) * kRmSamples, N, T, eta,
-                                          xT, ckpt, kck, traj, steps);
-  else
-    rm_morph_block<D, TRACE, 1, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, xT, ckpt, kck, traj,
-                                   steps);
+  const int warp = threadIdx.x >> 5;
+  float* xs = sm + 2 * kRmStageFloats + warp * (kRmWarpSamples * 8);   // [32 samples][8]: x, 0 .., 1
+  RmShare sh = rm_share(CS, nstage, sm + 2 * kRmStageFloats + kRmWarps * (kRmWarpSamples * 8));
+  const int64_t s0 = (int64_t)(blockIdx.x / CS) * kRmSamples + warp * kRmWarpSamples;
+  rm_load_rows<D>(x0, s0, N, 1.0f, xs);
+  for (int step = 0; step < T; ++step) {
+    rm_euler_step<D, TRACE, CS, kRmRows, CS == 1 ? kRmMorphUnroll : kRmUnroll<kRmRows>>(tab, sh, sm, xs, bias, eta, s0, N, step, traj, steps);
+    if (ckpt != nullptr && (step + 1) % kck == 0 && sh.crank == 0)
+      rm_store_rows<D>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
+  }
+  rm_leave<CS>(sh);
+  if (sh.crank > 0) return;
+  if (xT) rm_store_rows<D>(xs, s0, N, xT);
+  if (TRACE) rm_store_rows<D>(xs, s0, N, traj + (int64_t)T * N * D);
+}
+
+// the same on halves of 64 samples, one row tile a warp: few tiles with checkpoints
+template <int D>
+__global__ void __launch_bounds__(kRmWarps * 32, 4)
+k_morph_rff_halves(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N,
+                   int T, float eta, float* __restrict__ xT, float* __restrict__ ckpt, int kck) {
+  extern __shared__ __align__(16) float sm[];
+  rm_stage_init();
+  const int warp = threadIdx.x >> 5;
+  float* xs = sm + 2 * kRmStageFloats + warp * (16 * 8);
+  RmShare one = rm_share(1, nstage, nullptr);
+  const int64_t s0 = rm_first(blockIdx.x, 0) + warp * 16;
+  rm_load_rows<D, 1>(x0, s0, N, 1.0f, xs);
+  for (int step = 0; step < T; ++step) {
+    rm_euler_step<D, false, 1, 1>(tab, one, sm, xs, bias, eta, s0, N, step, nullptr, nullptr);
+    if (ckpt != nullptr && (step + 1) % kck == 0)
+      rm_store_rows<D, 1>(xs, s0, N, ckpt + (int64_t)((step + 1) / kck - 1) * N * D);
+  }
+  if (xT) rm_store_rows<D, 1>(xs, s0, N, xT);
 }
 
 // Weight-gradient pass at x (A fragments ah, al) with v = g (vh, vl), both
@@ -615,15 +626,14 @@ template <int D, int R>
 __device__ __forceinline__ void rm_vjp_block(float* sm, const float* __restrict__ tab, int nstage, float bias,
                                              const float* __restrict__ x0, int64_t first, int64_t N, int T, float eta,
                                              int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT,
-                                             float* __restrict__ g0, float* __restrict__ rows, int64_t M) {
+                                             float* __restrict__ g0, float* __restrict__ row, int64_t M) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   float* gs = sm + 2 * kRmStageFloats + warp * (kseg + 1) * ((R * 16) * 8);   // [32][8], column 7 = 0
   float* seg = gs + (R * 16) * 8;                                              // kseg x [32][8]
-  // weight gradient (rows != nullptr): this block's row of rows_[blocks][M + 1], warp partials, bias partials
+  // weight gradient (row != nullptr): this block's row of M + 1 floats, warp partials, bias partials
   float* part = sm + 2 * kRmStageFloats + kRmWarps * (kseg + 1) * ((R * 16) * 8);   // [4][128]
   float* gbw = part + kRmWarps * kRmStageKT * 8;                                        // [4]
-  float* row = rows ? rows + (int64_t)blockIdx.x * (M + 1) : nullptr;
   if (row)
     for (int64_t m = threadIdx.x; m <= M; m += blockDim.x) row[m] = 0.0f;
   float gb_acc = 0.0f;
@@ -653,7 +663,7 @@ __device__ __forceinline__ void rm_vjp_block(float* sm, const float* __restrict_
       rm_frags(gs, g, t, vh, vl);
       float G[R][4], P[R][4];
       u64 S[R][2];
-      rm_sweep<true>(tab, nstage, sm, ah, al, vh, vl, S, G, P);
+      rm_sweep<true, kRmUnroll<R>>(tab, nstage, sm, ah, al, vh, vl, S, G, P);
       float D1[R][2], D2[R][2], GD[R][2];
 #pragma unroll
       for (int r = 0; r < R; ++r)
@@ -717,14 +727,17 @@ template <int D>
 __global__ void __launch_bounds__(kRmWarps * 32, 3)
 k_vjp_rff_mma(const float* __restrict__ tab, int nstage, float bias, const float* __restrict__ x0, int64_t N, int T,
               float eta, int kseg, const float* __restrict__ ckpt, const float* __restrict__ gT, float* __restrict__ g0,
-              float* __restrict__ rows, int64_t M, unsigned n2) {
+              float* __restrict__ rows, int64_t M, unsigned n2, int64_t nrows, float* __restrict__ more) {
   extern __shared__ __align__(16) float sm[];
   rm_stage_init();
+  float* row = nullptr;
+  if (rows)
+    row = (int64_t)blockIdx.x < nrows ? rows + (int64_t)blockIdx.x * (M + 1)
+                                      : more + ((int64_t)blockIdx.x - nrows) * (M + 1);
   if (blockIdx.x < n2)
-    rm_vjp_block<D, kRmRows>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, rows,
-                             M);
+    rm_vjp_block<D, kRmRows>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, row, M);
   else
-    rm_vjp_block<D, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, rows, M);
+    rm_vjp_block<D, 1>(sm, tab, nstage, bias, x0, rm_first(blockIdx.x, n2), N, T, eta, kseg, ckpt, gT, g0, row, M);
 }
 
 static int rm_sms() {
@@ -818,16 +831,19 @@ static cudaError_t launch_rff_mma(const FieldArgs& fa, const float* x0, int64_t 
   // Checkpoints are where a VJP's replay starts, which runs one block per tile: their
   // sums are taken the same way, so that each segment ends where the next begins.
   const int cs = ckpt ? 1 : rm_cluster(tiles, nstage);
-  const RmDeal deal = cs > 1 ? RmDeal{0u, (unsigned)(tiles * cs)} : rm_deal(N, 4);
+  const RmDeal deal = rm_deal(N, 4);
+  if (cs == 1 && traj == nullptr && deal.n2 == 0)
+    return rm_launch(k_morph_rff_halves<D>, deal.blocks, 1, rm_smem_bytes(), st, tab, nstage, fa.bias, x0, N, T, eta,
+                     xT, ckpt, k);
   const size_t smem = rm_smem_bytes() + (cs > 1 ? kRmShareBytes : 0);
 #define PDMP_KERNEL(CS) (k_morph_rff_mma<D, true, CS>)
   if (traj != nullptr)
-    return PDMP_RM_LAUNCH(cs, deal.blocks, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, traj,
-                          steps, deal.n2);
+    return PDMP_RM_LAUNCH(cs, (unsigned)(tiles * cs), smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, traj,
+                          steps);
 #undef PDMP_KERNEL
 #define PDMP_KERNEL(CS) (k_morph_rff_mma<D, false, CS>)
-  return PDMP_RM_LAUNCH(cs, deal.blocks, smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, nullptr,
-                        nullptr, deal.n2);
+  return PDMP_RM_LAUNCH(cs, (unsigned)(tiles * cs), smem, st, PDMP_KERNEL, tab, nstage, fa.bias, x0, N, T, eta, xT, ckpt, k, nullptr,
+                        nullptr);
 #undef PDMP_KERNEL
 }
 
@@ -1084,7 +1100,7 @@ k_inverse_rff_mma(const float* __restrict__ tab, int nstage, float bias, const f
       rm_frags(ys, g, t, ah, al);
       float G[kRmRows][4], P[kRmRows][4];
       u64 S[kRmRows][2];
-      rm_sweep<false>(tab, nstage, sm, ah, al, ah, al, S, G, P);
+      rm_sweep<false, kRmUnroll<kRmRows>>(tab, nstage, sm, ah, al, ah, al, S, G, P);
       bool mv = false;
 #pragma unroll
       for (int r = 0; r < kRmRows; ++r)
@@ -1180,7 +1196,7 @@ cudaError_t stage_wait_selftest(const float* src, float* dst, long long limit, i
   return cudaGetLastError();
 }
 
-int64_t vjp_rff_mma_blocks(int64_t N) { return rm_deal(N, 3).blocks; }
+int64_t vjp_rff_mma_blocks(int64_t N) { return (N + kRmSamples - 1) / kRmSamples; }
 
 // the tensor-core VJP keeps a segment of states in shared memory: k <= 16
 size_t vjp_rff_mma_smem(int k) {
@@ -1198,13 +1214,20 @@ static cudaError_t launch_vjp_rff_mma(const FieldArgs& fa, const float* x0, int6
   const size_t smem = vjp_rff_mma_smem(k);
   cudaError_t e = cudaFuncSetAttribute(k_vjp_rff_mma<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const RmDeal deal = rm_deal(N, 3);
-  const unsigned blocks = deal.blocks;
-  k_vjp_rff_mma<D><<<blocks, kRmWarps * 32, smem, st>>>(tab, (int)(n_kt / kRmStageKT), fa.bias, x0, N, T, eta, k,
-                                                        ckpt, gT, g0, rows, fa.M, deal.n2);
+  // a row of d/dw a block: the workspace holds one a tile, and the halves' others
+  // go behind the table, which is made without the log-det's columns there (64
+  // floats a feature); more halves than that and the tiles go out whole
+  const int64_t tiles = vjp_rff_mma_blocks(N);
+  float* more = tab + n_kt * kRmKtFloats;
+  RmDeal deal = rm_deal(N, 3);
+  if (rows != nullptr && ((int64_t)deal.blocks - tiles) * (fa.M + 1) > n_kt * (kLdKtFloats - kRmKtFloats))
+    deal = RmDeal{(unsigned)tiles, (unsigned)tiles};
+  k_vjp_rff_mma<D><<<deal.blocks, kRmWarps * 32, smem, st>>>(tab, (int)(n_kt / kRmStageKT), fa.bias, x0, N, T, eta, k,
+                                                             ckpt, gT, g0, rows, fa.M, deal.n2, tiles, more);
   e = cudaGetLastError();
   if (e != cudaSuccess || rows == nullptr) return e;
-  return sum_vjp_rows(rows, (int64_t)blocks, fa.M + 1, gw, gbias, st);
+  return sum_vjp_rows(rows, min64(tiles, deal.blocks), fa.M + 1, gw, gbias, st, nullptr, more,
+                      (int64_t)deal.blocks > tiles ? deal.blocks - tiles : 0);
 }
 
 cudaError_t vjp_rff_mma(int d, const FieldArgs& fa, const float* x0, int64_t N, int T, float eta, int k,

@@ -252,11 +252,13 @@ k_morph_vjp(FieldArgs fa, const float* __restrict__ x0, int64_t N, int T, float 
 // sums the per-block rows in block order: out[m] = sum_b rows[b][m], m <= M
 // (perm: NULL, or the feature of each row position)
 __global__ void k_sum_rows(const float* __restrict__ rows, int64_t nrows, int64_t width, float* __restrict__ gw,
-                           float* __restrict__ gbias, const int32_t* __restrict__ perm) {
+                           float* __restrict__ gbias, const int32_t* __restrict__ perm,
+                           const float* __restrict__ more, int64_t nmore) {
   int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= width) return;
   double acc = 0.0;   // hundreds of rows: FP64 costs nothing beside their loads
   for (int64_t b = 0; b < nrows; ++b) acc += (double)rows[b * width + m];
+  for (int64_t b = 0; b < nmore; ++b) acc += (double)more[b * width + m];
   if (m + 1 < width) {
     if (gw) gw[perm ? perm[m] : m] = (float)acc;
   } else if (gbias) {
@@ -265,8 +267,8 @@ __global__ void k_sum_rows(const float* __restrict__ rows, int64_t nrows, int64_
 }
 
 cudaError_t sum_vjp_rows(const float* rows, int64_t nrows, int64_t width, float* gw, float* gbias, cudaStream_t st,
-                         const int32_t* perm) {
-  k_sum_rows<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(rows, nrows, width, gw, gbias, perm);
+                         const int32_t* perm, const float* more, int64_t nmore) {
+  k_sum_rows<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(rows, nrows, width, gw, gbias, perm, more, nmore);
   return cudaGetLastError();
 }
 
