@@ -250,7 +250,7 @@ pdmp_status pdmp_graph_destroy(void* graph_exec);
  *            128), W3 (128 x 128), W4 (3 x 128), each [out][in] row-major;
  *   b        FP32 biases, PDMP_MLP_NB floats: b1, b2, b3 (128 each), b4 (3);
  *   W_bf16   BF16 copy of W (same layout), the weights the kernels use;
- *   Wt_bf16  BF16 transposes of W2 and W3 (2 x 128 x 128), for the backward;
+ *   Wt_bf16  BF16 transposes of W2 and W3 (2 x 128 x 128), for the FP32-activation gradient's backward;
  *   adam     Adam moments: m_W, v_W (PDMP_MLP_NW each), m_b, v_b (PDMP_MLP_NB
  *            each); zero before the first step.
  * Matrix products run on the tensor cores in BF16 with FP32 accumulation,

@@ -779,7 +779,8 @@ static int rm_cluster(int64_t tiles, int nstage) {
 // Tiles past the last full wave (per_sm blocks on every SM) go out as halves, if
 // the halves fit on the GPU at once: a half is over in about 0.65 of a tile's
 // time, and up to twice as many SMs take part.  Not where the tiles would be one to an
-// SM behind full waves (two halves to an SM are then no faster).  Measured
+// SM behind full waves (two halves to an SM are then no faster).  Measured, with
+// k tiles unrolled by two (log-det one)
 // (ms, M = 4096, T = 20, whole tiles / dealt; per_sm 3): VJP with d/dw and its
 // forward of 2000 samples 7.33 / 5.42, 25,000 10.3 / 8.16, 65,537 19.6 / 18.0;
 // log-det 3.11 / 2.37, 4.64 / 3.75, 8.91 / 8.06; all in halves is slower from
